@@ -129,7 +129,7 @@ cudaError_t set_coefficients(sl_ctx *c, const sl_field *drift, const sl_field *d
         e = stage_nodal(c, drift, m.dim * V, nif, du);
         if (e == cudaSuccess) e = stage_nodal(c, diffusion, V, nif, dD);
     }
-    ++c->fields_version;  // the 2D advance coefficients are formed again at the next step
+    ++c->fields_version;  // the advance coefficients are formed again at the next step
     if (e == cudaSuccess)
         e = sl::launch_init_fields(m, du, dD, to_dev(phi0), phi0_nodal_dev, c->xi, c->nodeU, c->nodeB, c->nodeDiv,
                                    c->faceU, c->faceB, write_state ? c->Q : nullptr, c->M * c->ncomp,
@@ -255,16 +255,19 @@ int refresh_bounds(sl_ctx *c)
 }  // namespace
 
 namespace sl {
-// The 2D advance coefficients for step size dt, formed on the context's
-// stream when the step size or the fields changed since the last time.
-cudaError_t ensure_coef2d(sl_ctx *c, double dt)
+// The advance coefficients for step size dt, formed on the context's stream
+// when the step size or the fields changed since the last time.
+cudaError_t ensure_coef(sl_ctx *c, double dt)
 {
-    if (c->m.dim != 2 || (c->coef2d_dt == dt && c->coef2d_version == c->fields_version)) return cudaSuccess;
-    const cudaError_t e = launch_coef2d(c->nodeU, c->nodeB, c->nodeDiv, (long long)c->m.E * c->m.n, dt,
-                                        4.0 / c->m.h[0], 4.0 / c->m.h[1], c->precision == SL_FP64, c->coef2d, c->st);
+    if (c->coef_dt == dt && c->coef_version == c->fields_version) return cudaSuccess;
+    const bool fp64 = c->precision == SL_FP64;
+    const cudaError_t e =
+        c->m.dim == 1 ? launch_coef1d(c->m, c->nodeU, c->nodeB, c->nodeDiv, c->faceU, c->faceB, dt, fp64, c->coef, c->st)
+                      : launch_coef2d(c->nodeU, c->nodeB, c->nodeDiv, (long long)c->m.E * c->m.n, dt, 4.0 / c->m.h[0],
+                                      4.0 / c->m.h[1], fp64, c->coef, c->st);
     if (e == cudaSuccess) {
-        c->coef2d_dt = dt;
-        c->coef2d_version = c->fields_version;
+        c->coef_dt = dt;
+        c->coef_version = c->fields_version;
     }
     return e;
 }
@@ -329,7 +332,7 @@ void sl_free(sl_ctx *c)
     sl::ctx_free(c, c->faces2d);
     sl::ctx_free(c, c->tab2d);
     sl::ctx_free(c, c->alpha2d);
-    sl::ctx_free(c, c->coef2d);
+    sl::ctx_free(c, c->coef);
     sl::ctx_free(c, c->fb2d);
     sl::ctx_free(c, c->fbcount2d);
     sl::ctx_free(c, c->slots2d);
@@ -423,13 +426,14 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
               dalloc(c, &c->psq, size_t(nc) * ncomp * V) == cudaSuccess &&
               dalloc(c, &c->mean_tmp, ncomp * V) == cudaSuccess && dalloc(c, &c->m2_tmp, ncomp * V) == cudaSuccess &&
               dalloc(c, &c->err, 1) == cudaSuccess &&
+              sl::ctx_alloc(c, &c->coef, (dim == 1 ? size_t(3) * V + 2 * (m.E + 1) : size_t(5) * V) *
+                                             (precision == SL_FP64 ? 8 : 4)) == cudaSuccess &&
               (dim == 1 || (dalloc(c, &c->faceUhi, size_t(m.K[0] + m.K[1]) * N) == cudaSuccess &&
                             dalloc(c, &c->faceBhi, size_t(m.K[0] + m.K[1]) * N) == cudaSuccess));
     if (ok && dim == 2)
         ok = sl::ctx_alloc(c, &c->faces2d, size_t(M) * ncomp * m.E * 4 * N * c->state_elem) == cudaSuccess &&
              dalloc(c, &c->tab2d, size_t(N) * N + 5 * N) == cudaSuccess &&
              sl::ctx_alloc(c, &c->alpha2d, size_t(M) * ncomp * V * (precision == SL_FP64 ? 8 : 4)) == cudaSuccess &&
-             sl::ctx_alloc(c, &c->coef2d, size_t(5) * V * (precision == SL_FP64 ? 8 : 4)) == cudaSuccess &&
              sl::ctx_alloc(c, reinterpret_cast<void **>(&c->fb2d), size_t(M) * m.E) == cudaSuccess &&
              sl::ctx_alloc(c, reinterpret_cast<void **>(&c->fbcount2d), 2 * sizeof(unsigned long long)) ==
                  cudaSuccess &&
@@ -620,6 +624,7 @@ int sl_step(sl_ctx *c, double dt, int steps)
         if (c->reseed_every > 0)  // stop at the next reseed point
             n = int(std::min<long long>(n, c->reseed_every - c->step % c->reseed_every));
         cudaError_t e = sl::launch_wiener(c->seed, c->step, c->sample0, n, c->M, dim, sqrt_dt, c->dW, c->st);
+        if (e == cudaSuccess) e = sl::ensure_coef(c, dt);
         if (e != cudaSuccess) return fail_cuda(c);
         std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
         if (c->profiling) {
@@ -636,18 +641,12 @@ int sl_step(sl_ctx *c, double dt, int steps)
             a.C = c->C;
             a.T = c->T;
             a.nsteps = n;
-            a.dt = dt;
-            a.h = m.h[0];
             a.inv_w2 = c->inv_w2;
             a.periodic = c->periodic;
             a.ncomp = c->ncomp;
             a.ghost = c->periodic ? nullptr : c->ghost + c->ghost_w * (c->step - c->ghost_base);
             a.xi = c->xi;
-            a.nodeU = c->nodeU;
-            a.nodeB = c->nodeB;
-            a.nodeDiv = c->nodeDiv;
-            a.faceU = c->faceU;
-            a.faceB = c->faceB;
+            a.coef = c->coef;
             a.dW = c->dW;
             a.Q = c->Q;
             a.err = c->err;
@@ -685,8 +684,7 @@ int sl_step(sl_ctx *c, double dt, int steps)
             a.Q = c->Q;
             a.faces = c->faces2d;
             a.alpha = c->alpha2d;
-            a.coef = c->coef2d;
-            if (sl::ensure_coef2d(c, dt) != cudaSuccess) return fail_cuda(c);
+            a.coef = c->coef;
             a.err = c->err;
             a.chunk = c->launch_chunk;
             a.g0 = a.g1 = 0;

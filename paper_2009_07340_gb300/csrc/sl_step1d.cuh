@@ -198,15 +198,16 @@ __device__ __forceinline__ void step1d_body(const Step1DArgs &a, const int slot)
     const int T = a.T, S = a.S, K = a.K;
     constexpr int NP = (N + 3) & ~3;            // padded row of the Z table
     // face pairs first (8-byte aligned for any S, T), then the 16-byte
-    // aligned Z table (4 S T faces of 8 bytes = a multiple of 32 bytes)
+    // aligned Z table (4 S T faces of 8 bytes = a multiple of 32 bytes; FP64
+    // only: the FP32 kernels' node tables are compile-time constants)
     FaceT *sface = reinterpret_cast<FaceT *>(smem_raw);           // [2 buf][2 side][NCOMP][S][T]
     R *sZ = reinterpret_cast<R *>(smem_raw + sizeof(FaceT) * 4 * NCOMP * S * T);  // [N][NP] zeta_i - zeta_m
-    R *sal = sZ + N * NP;                      // [N][T] 4 u dt / h
+    R *sF0 = sZ + (kPair ? 0 : N * NP);        // [N] 0 - zeta_m
+    R *sF1 = sF0 + (kPair ? 0 : N);            // [N] 4 - zeta_m
+    R *sal = sF1 + (kPair ? 0 : N);            // [N][T] 4 u dt / h
     R *sbe = sal + N * T;                      // [N][T] 4 b / h
     R *sga = sbe + N * T;                      // [N][T] dt du/dx
-    R *sF0 = sga + N * T;                      // [N] 0 - zeta_m
-    R *sF1 = sF0 + N;                          // [N] 4 - zeta_m
-    R *sfa = sF1 + N;                          // [T + 1] u dt at the interfaces k0 .. k1
+    R *sfa = sga + N * T;                      // [T + 1] u dt at the interfaces k0 .. k1
     R *sfb = sfa + (T + 1);                    // [T + 1] sqrt(2 D)
     constexpr NodeTab1D<N> kTab{};
     auto F0 = [&](int m) -> R { if constexpr (kPair) return kTab.f0[m]; else return sF0[m]; };
@@ -220,31 +221,28 @@ __device__ __forceinline__ void step1d_body(const Step1DArgs &a, const int slot)
     const int Kc = k1 - k0;
 
     // dt-dependent coefficient tables of this CTA's elements
+    const R *cf = static_cast<const R *>(a.coef);
     for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
         const int j = idx / T, kl = idx - j * T;
-        double al = 0.0, be = 0.0, ga = 0.0;  // idle slots: unmoved nodes
-        if (kl < Kc) {
-            const int k = k0 + kl;
-            al = 4.0 * a.nodeU[k * N + j] * a.dt / a.h;
-            be = 4.0 * a.nodeB[k * N + j] / a.h;
-            ga = a.dt * a.nodeDiv[k * N + j];
+        const bool own = kl < Kc;  // idle slots: unmoved nodes
+        const R *c = cf + j * K + k0 + kl;
+        sal[idx] = own ? c[0] : R(0);
+        sbe[idx] = own ? c[N * K] : R(0);
+        sga[idx] = own ? c[2 * N * K] : R(0);
+    }
+    for (int idx = threadIdx.x; idx <= Kc; idx += blockDim.x) {  // interface f: left face of element f
+        sfa[idx] = cf[3 * N * K + k0 + idx];
+        sfb[idx] = cf[3 * N * K + K + 1 + k0 + idx];
+    }
+    if constexpr (!kPair) {
+        for (int idx = threadIdx.x; idx < N * NP; idx += blockDim.x) {
+            const int i = idx / NP, m = idx - i * NP;
+            sZ[idx] = m < N ? R(4.0 * (a.xi[i] - a.xi[m])) : R(0);
         }
-        sal[idx] = R(al);
-        sbe[idx] = R(be);
-        sga[idx] = R(ga);
-    }
-    for (int idx = threadIdx.x; idx < N * NP; idx += blockDim.x) {
-        const int i = idx / NP, m = idx - i * NP;
-        sZ[idx] = m < N ? R(4.0 * (a.xi[i] - a.xi[m])) : R(0);
-    }
-    for (int idx = threadIdx.x; idx <= Kc; idx += blockDim.x) {
-        const int f = a.periodic ? (k0 + idx) % K : k0 + idx;  // interface f: left face of element f
-        sfa[idx] = R(a.faceU[f] * a.dt);
-        sfb[idx] = R(a.faceB[f]);
-    }
-    if (threadIdx.x < N) {
-        sF0[threadIdx.x] = R(-4.0 * a.xi[threadIdx.x]);
-        sF1[threadIdx.x] = R(4.0 * (1.0 - a.xi[threadIdx.x]));
+        if (threadIdx.x < N) {
+            sF0[threadIdx.x] = R(-4.0 * a.xi[threadIdx.x]);
+            sF1[threadIdx.x] = R(4.0 * (1.0 - a.xi[threadIdx.x]));
+        }
     }
 
     const int sl = threadIdx.x / T;
@@ -594,7 +592,8 @@ size_t step1d_smem_bytes_t(int N, int S, int T, int ncomp = 1)
 {
     using R = typename Prec1D<MODE>::R;
     const int NP = (N + 3) & ~3;
-    return sizeof(R) * (size_t(N) * NP + size_t(3) * N * T + 2 * N + 2 * (T + 1)) + size_t(8) * 4 * ncomp * S * T;
+    const size_t tab = sizeof(R) == 8 ? size_t(N) * NP + 2 * N : 0;
+    return sizeof(R) * (tab + size_t(3) * N * T + 2 * (T + 1)) + size_t(8) * 4 * ncomp * S * T;
 }
 
 template <int N, int MODE>

@@ -44,12 +44,10 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int T = a.T, S = a.S, K = a.K;
     float2 *sface = reinterpret_cast<float2 *>(smem_raw);                 // [2 buf][2 side][S][T] pairs
-    float *sZ = reinterpret_cast<float *>(sface + 4 * S * T);             // [N][NP] zeta_j - zeta_m
-    float2 *sal = reinterpret_cast<float2 *>(sZ + N * NP);                // [NH][T] 4 u dt / h
+    float2 *sal = sface + 4 * S * T;                                      // [NH][T] 4 u dt / h
     float2 *sbe = sal + NH * T;                                           // [NH][T] 4 b / h
     float2 *sng = sbe + NH * T;                                           // [NH][T] -dt du/dx
-    float2 *sF = sng + NH * T;                                            // [N] (0 - zeta_m, 4 - zeta_m)
-    float *sfa = reinterpret_cast<float *>(sF + N);                       // [T + 1] u dt at interfaces
+    float *sfa = reinterpret_cast<float *>(sng + NH * T);                 // [T + 1] u dt at interfaces
     float *sfb = sfa + (T + 1);                                           // [T + 1] sqrt(2 D)
     // node tables as compile-time constants (see NodeTab1D): rows of Z padded
     // with zeros past N, face pairs (0 - zeta_m, 4 - zeta_m)
@@ -67,37 +65,26 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
     const int k1 = int((long long)K * (rank + 1) / C);
     const int Kc = k1 - k0;
 
+    const float *cf = static_cast<const float *>(a.coef);
     for (int idx = threadIdx.x; idx < NH * T; idx += blockDim.x) {
         const int p = idx / T, kl = idx - p * T;
         float v[3][2];
         for (int l = 0; l < 2; ++l) {
             const int j = 2 * p + l;
-            double al = 0.0, be = 0.0, ga = 0.0;
-            if (kl < Kc && j < N) {
-                const int k = k0 + kl;
-                al = 4.0 * a.nodeU[k * N + j] * a.dt / a.h;
-                be = 4.0 * a.nodeB[k * N + j] / a.h;
-                ga = a.dt * a.nodeDiv[k * N + j];
-            }
-            v[0][l] = float(al);
-            v[1][l] = float(be);
-            v[2][l] = float(-ga);
+            const bool own = kl < Kc && j < N;
+            const float *c = cf + j * K + k0 + kl;
+            v[0][l] = own ? c[0] : 0.f;
+            v[1][l] = own ? c[N * K] : 0.f;
+            v[2][l] = own ? -c[2 * N * K] : 0.f;
         }
         sal[idx] = make_float2(v[0][0], v[0][1]);
         sbe[idx] = make_float2(v[1][0], v[1][1]);
         sng[idx] = make_float2(v[2][0], v[2][1]);
     }
-    for (int idx = threadIdx.x; idx < N * NP; idx += blockDim.x) {
-        const int j = idx / NP, m = idx - j * NP;
-        sZ[idx] = m < N ? float(4.0 * (a.xi[j] - a.xi[m])) : 0.f;
+    for (int idx = threadIdx.x; idx <= Kc; idx += blockDim.x) {  // interface f: left face of element f
+        sfa[idx] = cf[3 * N * K + k0 + idx];
+        sfb[idx] = cf[3 * N * K + K + 1 + k0 + idx];
     }
-    for (int idx = threadIdx.x; idx <= Kc; idx += blockDim.x) {
-        const int f = a.periodic ? (k0 + idx) % K : k0 + idx;  // K: the boundary x = hi
-        sfa[idx] = float(a.faceU[f] * a.dt);
-        sfb[idx] = float(a.faceB[f]);
-    }
-    if (threadIdx.x < N)
-        sF[threadIdx.x] = make_float2(float(-4.0 * a.xi[threadIdx.x]), float(4.0 * (1.0 - a.xi[threadIdx.x])));
 
     const int sl = threadIdx.x / T;
     const int kl = threadIdx.x - sl * T;
@@ -374,9 +361,8 @@ __global__ void __launch_bounds__(kMaxThreads1D, SL1D_FP32_MIN_BLOCKS) sl1d_step
 template <int MODE>
 size_t step1d_f2_smem_bytes(int N, int S, int T)
 {
-    const int NE = N + (N & 1), NH = NE / 2, NP = (NE + 3) & ~3;
-    return sizeof(float2) * (size_t(4) * S * T) + sizeof(float) * size_t(N) * NP +
-           sizeof(float2) * (size_t(3) * NH * T + N) + sizeof(float) * 2 * (T + 1);
+    const int NE = N + (N & 1), NH = NE / 2;
+    return sizeof(float2) * (size_t(4) * S * T + size_t(3) * NH * T) + sizeof(float) * 2 * (T + 1);
 }
 
 template <int N, int MODE>
