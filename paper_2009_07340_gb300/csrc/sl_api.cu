@@ -131,10 +131,12 @@ cudaError_t set_coefficients(sl_ctx *c, const sl_field *drift, const sl_field *d
     }
     ++c->fields_version;  // the advance coefficients are formed again at the next step
     if (e == cudaSuccess)
-        e = sl::launch_init_fields(m, du, dD, to_dev(phi0), phi0_nodal_dev, c->xi, c->nodeU, c->nodeB, c->nodeDiv,
-                                   c->faceU, c->faceB, write_state ? c->Q : nullptr, c->M * c->ncomp,
-                                   c->precision == SL_FP64, c->st);  // [M][ncomp] fields of E n values
-    if (e == cudaSuccess && m.dim == 2) e = sl::launch_init_faces_hi(m, du, dD, c->faceUhi, c->faceBhi, c->st);
+        e = sl::launch_init_fields(m, du, dD, to_dev(phi0), phi0_nodal_dev, c->ref, c->nodeU, c->nodeB, c->nodeDiv,
+                                   c->faceU, c->faceB, write_state ? c->mean_tmp : nullptr, c->st);
+    if (e == cudaSuccess && write_state)  // every one of the [M][ncomp] fields of E n values
+        e = sl::launch_reseed(c->Q, c->precision == SL_FP64, c->M * c->ncomp, V, c->mean_tmp, c->st);
+    if (e == cudaSuccess && m.dim == 2 && !c->periodic)  // read on Dirichlet boundaries only
+        e = sl::launch_init_faces_hi(m, du, dD, c->ref, c->faceUhi, c->faceBhi, c->st);
     if (!device_tables) {
         unstage_nodal(c, du);
         unstage_nodal(c, dD);
@@ -317,6 +319,7 @@ void sl_free(sl_ctx *c)
     sl::ctx_free(c, c->faceUhi);
     sl::ctx_free(c, c->faceBhi);
     sl::ctx_free(c, c->xi);
+    sl::ctx_free(c, c->ref);
     sl::ctx_free(c, c->nodeU);
     sl::ctx_free(c, c->nodeB);
     sl::ctx_free(c, c->nodeDiv);
@@ -418,7 +421,7 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
     const int nf = dim == 1 ? m.E + 1 : 2 * m.E * N;  // 1D: interfaces 0..K
     c->mom_chunk = 64;
     const int nc = (M + c->mom_chunk - 1) / c->mom_chunk;
-    bool ok = dalloc(c, &c->xi, N) == cudaSuccess && dalloc(c, &c->nodeU, size_t(dim) * V) == cudaSuccess &&
+    bool ok = dalloc(c, &c->xi, N) == cudaSuccess && dalloc(c, &c->ref, size_t(N) * N + 3 * N) == cudaSuccess && dalloc(c, &c->nodeU, size_t(dim) * V) == cudaSuccess &&
               dalloc(c, &c->nodeB, V) == cudaSuccess && dalloc(c, &c->nodeDiv, V) == cudaSuccess &&
               dalloc(c, &c->faceU, nf) == cudaSuccess && dalloc(c, &c->faceB, nf) == cudaSuccess &&
               sl::ctx_alloc(c, &c->Q, size_t(M) * ncomp * V * c->state_elem) == cudaSuccess &&
@@ -456,6 +459,7 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
         }
     }
     cudaError_t e = cudaMemsetAsync(c->err, 0, sizeof(int), c->st);
+    if (e == cudaSuccess) e = sl::launch_ref_tables(N, c->ref, c->xi, c->st);
     if (e == cudaSuccess) e = set_coefficients(c, drift, diffusion, phi0, nodal_dev, true);  // every sample phi0
     sl::ctx_free(c, nodal_dev);
     if (e != cudaSuccess || refresh_bounds(c) != SL_OK) {

@@ -169,10 +169,12 @@ cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double
                           double s4x, double s4y, bool fp64, void *out, cudaStream_t st);
 // Host-side node tables of a 2D order (Step2DArgs::tab) from the nodes xi[N].
 void node_tables2d(int N, const double *xi, double *tab);
+// Reference tables of order N (derivative matrix, face values, nodes) and the nodes alone.
+cudaError_t launch_ref_tables(int N, double *ref, double *xi, cudaStream_t st);
+// Node and face coefficients; phi (or null): the initial value at every node.
 cudaError_t launch_init_fields(const Mesh &m, const FieldDev &u, const FieldDev &D, const FieldDev &phi0,
-                               const double *phi0_nodal_dev, double *xi, double *nodeU, double *nodeB,
-                               double *nodeDiv, double *faceU, double *faceB, void *Q, int M,
-                               int state_is_double, cudaStream_t st);
+                               const double *phi0_nodal_dev, const double *ref, double *nodeU, double *nodeB,
+                               double *nodeDiv, double *faceU, double *faceB, double *phi, cudaStream_t st);
 cudaError_t launch_wiener(unsigned long long seed, long long step0, long long sample0, int nsteps, int M, int dim,
                           double sqrt_dt, double *out, cudaStream_t st);
 cudaError_t launch_moments(const void *Q, int state_is_double, int M, long long V, int chunk,
@@ -187,8 +189,8 @@ cudaError_t launch_moments_combine(const double *psum, const double *psq, int nc
 cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, int B, double lo, double hi,
                        unsigned int *counts, cudaStream_t st);
 // 2D coefficients on the faces x = hi ([Ky][N], u_x) and y = hi ([Kx][N], u_y).
-cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, double *faceUhi, double *faceBhi,
-                                 cudaStream_t st);
+cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, const double *ref,
+                                 double *faceUhi, double *faceBhi, cudaStream_t st);
 // Every sample set to `mean` (Eq. re-seed).
 cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, cudaStream_t st);
 
@@ -241,6 +243,7 @@ struct sl_ctx {
     double dtmax = 0.0;   // Eq. (1d_timestep) with the smallest node gap
     double dtedge = 0.0;  // the same with the first node's distance to the element face
     // device memory owned by the context
+    double *ref = nullptr;  // reference tables of the order [N N + 3 N] (launch_ref_tables)
     double *xi = nullptr, *nodeU = nullptr, *nodeB = nullptr, *nodeDiv = nullptr;
     double *faceU = nullptr, *faceB = nullptr;
     void *Q = nullptr;

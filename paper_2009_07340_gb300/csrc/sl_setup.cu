@@ -17,16 +17,16 @@ namespace sl {
 // (Eq. gaussquad with (i+1/2)/N, interleaved with the Lobatto nodes).
 __device__ __forceinline__ double gauss_node(int i, int N) { return 0.5 * (1.0 - cospi((i + 0.5) / N)); }
 
-// d h_m / d xi at x for the Lagrange basis on the Gauss nodes (product rule).
-__device__ double lagrange_deriv(int N, int m, double x)
+// d h_m / d xi at x for the Lagrange basis on the Gauss nodes g (product rule).
+__device__ double lagrange_deriv(int N, int m, double x, const double *g)
 {
     double sum = 0.0;
-    const double xm = gauss_node(m, N);
+    const double xm = g[m];
     for (int k = 0; k < N; ++k) {
         if (k == m) continue;
-        double v = 1.0 / (xm - gauss_node(k, N));
+        double v = 1.0 / (xm - g[k]);
         for (int l = 0; l < N; ++l)
-            if (l != m && l != k) v *= (x - gauss_node(l, N)) / (xm - gauss_node(l, N));
+            if (l != m && l != k) v *= (x - g[l]) / (xm - g[l]);
         sum += v;
     }
     return sum;
@@ -52,13 +52,13 @@ __device__ double diffusion_at(const FieldDev &f, double x, double y)
     }
 }
 
-// h_l(x): the Lagrange basis polynomial l on the Gauss nodes (product form).
-__device__ double lagrange_at(int N, int l, double x)
+// h_l(x): the Lagrange basis polynomial l on the Gauss nodes g (product form).
+__device__ double lagrange_at(int N, int l, double x, const double *g)
 {
-    const double xl = gauss_node(l, N);
+    const double xl = g[l];
     double v = 1.0;
-    for (int k = 0; k < N; ++k)
-        if (k != l) v *= (x - gauss_node(k, N)) / (xl - gauss_node(k, N));
+    for (int m = 0; m < N; ++m)
+        if (m != l) v *= (x - g[m]) / (xl - g[m]);
     return v;
 }
 
@@ -80,15 +80,50 @@ __device__ __forceinline__ double node_diffusion(const FieldDev &f, long long v,
     return f.kind == SL_D_NODAL ? f.nodal[v] : diffusion_at(f, x, y);
 }
 
-// Trace of element e's nodal interpolant of vals ([E][n]) on its face
-// xi_dir = side, at the face's Gauss point pt (0 in 1D).
-__device__ double trace_of(const Mesh &m, const double *vals, int e, int dir, double side, int pt)
+// Reference tables of an order (ref [N N + 3 N]): d h_m / d xi at node i
+// ([i][m]), h_l(0), h_l(1), the nodes.  Formed once per context.  The setup
+// kernels used to evaluate these inside every node's and face's loops (an
+// O(N^3) product with two FP64 cospi per factor and node): new fields on
+// 32 x 32 elements of N = 5 before each of two steps of 64 samples made the
+// pair of steps take 2.77 ms, now 0.85.
+struct RefTab {
+    const double *diff, *at0, *at1, *xi;
+    __host__ __device__ RefTab(const double *ref, int N) : diff(ref), at0(ref + N * N), at1(at0 + N), xi(at1 + N) {}
+};
+
+// One block per node i (N <= 32 threads): row i of the derivative matrix;
+// block 0 also the face values and the nodes.
+__global__ void ref_tables_kernel(int N, double *ref, double *xi)
+{
+    __shared__ double x[kMaxN];
+    const int i = blockIdx.x, m = threadIdx.x;
+    if (m < N) x[m] = gauss_node(m, N);
+    __syncthreads();
+    if (m >= N) return;
+    ref[i * N + m] = lagrange_deriv(N, m, x[i], x);
+    if (i == 0) {
+        ref[N * N + m] = lagrange_at(N, m, 0.0, x);
+        ref[N * N + N + m] = lagrange_at(N, m, 1.0, x);
+        ref[N * N + 2 * N + m] = x[m];
+        xi[m] = x[m];
+    }
+}
+
+cudaError_t launch_ref_tables(int N, double *ref, double *xi, cudaStream_t st)
+{
+    ref_tables_kernel<<<N, 32, 0, st>>>(N, ref, xi);
+    return cudaGetLastError();
+}
+
+// Trace of element e's nodal interpolant of vals ([E][n]) on its face with
+// basis values h there (h_l(0) or h_l(1)), at the face's Gauss point pt (0 in 1D).
+__device__ double trace_of(const Mesh &m, const double *vals, int e, int dir, const double *h, int pt)
 {
     const int N = m.N;
     double s = 0.0;
     for (int l = 0; l < N; ++l) {
         const int node = m.dim == 1 ? l : (dir == 0 ? pt * N + l : l * N + pt);
-        s += lagrange_at(N, l, side) * vals[(long long)e * m.n + node];
+        s += h[l] * vals[(long long)e * m.n + node];
     }
     return s;
 }
@@ -99,8 +134,8 @@ __device__ double trace_of(const Mesh &m, const double *vals, int e, int dir, do
 // [K1+1][K0][N]), else the mean of the traces of the elements on both sides,
 // the inside one alone at a Dirichlet boundary.  On a periodic mesh
 // interface K is interface 0.
-__device__ double iface_nodal(const Mesh &m, const double *vals, const double *face, int dir, int line, int idx,
-                              int pt)
+__device__ double iface_nodal(const Mesh &m, const RefTab &ref, const double *vals, const double *face, int dir,
+                              int line, int idx, int pt)
 {
     const int K = m.K[dir];
     if (m.periodic && idx == K) idx = 0;
@@ -113,8 +148,8 @@ __device__ double iface_nodal(const Mesh &m, const double *vals, const double *f
     const int kl = (idx - 1 + K) % K;
     const int el = dir == 0 ? line * m.K[0] + kl : kl * m.K[0] + line;
     const int er = dir == 0 ? line * m.K[0] + idx : idx * m.K[0] + line;
-    const double l = has_l ? trace_of(m, vals, el, dir, 1.0, pt) : 0.0;
-    const double r = has_r ? trace_of(m, vals, er, dir, 0.0, pt) : 0.0;
+    const double l = has_l ? trace_of(m, vals, el, dir, ref.at1, pt) : 0.0;
+    const double r = has_r ? trace_of(m, vals, er, dir, ref.at0, pt) : 0.0;
     if (has_l && has_r) return 0.5 * (l + r);
     return has_l ? l : r;
 }
@@ -122,11 +157,11 @@ __device__ double iface_nodal(const Mesh &m, const double *vals, const double *f
 // Normal drift u_dir and sqrt(2 D) at an interface point at (x, y); nodal
 // kinds through iface_nodal, a derived D clipped at 0 (D >= 0 on the nodes
 // does not bound the interpolant's trace).
-__device__ void face_fields(const FieldDev &fu, const FieldDev &fD, const Mesh &m, int dir, int line, int idx,
-                            int pt, double x, double y, double &un, double &b)
+__device__ void face_fields(const FieldDev &fu, const FieldDev &fD, const Mesh &m, const RefTab &ref, int dir,
+                            int line, int idx, int pt, double x, double y, double &un, double &b)
 {
     if (fu.kind == SL_U_NODAL) {
-        un = iface_nodal(m, fu.nodal + (long long)dir * m.E * m.n, fu.face, dir, line, idx, pt);
+        un = iface_nodal(m, ref, fu.nodal + (long long)dir * m.E * m.n, fu.face, dir, line, idx, pt);
     } else {
         double ux, uy;
         drift_at(fu, x, y, ux, uy);
@@ -134,7 +169,7 @@ __device__ void face_fields(const FieldDev &fu, const FieldDev &fD, const Mesh &
     }
     double D;
     if (fD.kind == SL_D_NODAL) {
-        D = iface_nodal(m, fD.nodal, fD.face, dir, line, idx, pt);
+        D = iface_nodal(m, ref, fD.nodal, fD.face, dir, line, idx, pt);
         if (fD.face && fD.err && !(D >= 0.0)) atomicOr(fD.err, 4);  // a given value below 0
         D = fmax(D, 0.0);  // a derived trace may undershoot
     } else {
@@ -175,10 +210,6 @@ __device__ double phi0_at(const FieldDev &f, const Mesh &m, double x, double y)
     }
 }
 
-// One thread per node (e, p): physical coordinates, drift, sqrt(2D), the
-// divergence of the drift by spectral differentiation along the element's
-// grid lines (the paper takes du/dx from the DSEM solver, Section 5.2), and
-// the initial value written to every sample.
 __device__ __forceinline__ void store_state(double *Q, long long i, double v) { Q[i] = v; }
 __device__ __forceinline__ void store_state(float2 *Q, long long i, double v)
 {
@@ -192,87 +223,84 @@ __device__ __forceinline__ double load_state(const float2 *Q, long long i)
     return double(v.x) + double(v.y);
 }
 
-template <typename State>
-__global__ void init_nodes_kernel(Mesh m, FieldDev fu, FieldDev fD, FieldDev fphi, const double *phi0_nodal,
-                                  double *xi, double *nodeU, double *nodeB, double *nodeDiv, State *Q, int M)
+// One thread per node (e, p), a block per `epb` elements: physical
+// coordinates, drift, sqrt(2D), the initial value, and the divergence of the
+// drift by spectral differentiation along the element's grid lines (the paper
+// takes du/dx from the DSEM solver, Section 5.2), from the element's own
+// node values in shared memory.
+constexpr int kInitThreads = 256;  // >= 144, the nodes of the largest 2D element
+
+__global__ void __launch_bounds__(kInitThreads)
+    init_nodes_kernel(Mesh m, FieldDev fu, FieldDev fD, FieldDev fphi, const double *phi0_nodal, const double *ref,
+                      double *nodeU, double *nodeB, double *nodeDiv, double *phi, int epb)
 {
+    __shared__ double su[2][kInitThreads];
+    const RefTab r(ref, m.N);
     const long long V = (long long)m.E * m.n;
-    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < m.N && blockIdx.x == 0) xi[v] = gauss_node(int(v), m.N);
-    if (v >= V) return;
-    const int e = int(v / m.n), p = int(v % m.n);
-    const int N = m.N;
-    const int kx = e % m.K[0], ky = e / m.K[0];
-    const int i = p % N, j = p / N;
-    const double x = m.lo[0] + (kx + gauss_node(i, N)) * m.h[0];
-    const double y = m.dim == 2 ? m.lo[1] + (ky + gauss_node(j, N)) * m.h[1] : 0.0;
-    double ux, uy;
-    node_drift(fu, m, v, x, y, ux, uy);
-    nodeU[v] = ux;
-    if (m.dim == 2) nodeU[V + v] = uy;
-    const double Dv = node_diffusion(fD, v, x, y);
-    if (fD.err && !(Dv >= 0.0)) atomicOr(fD.err, 4);  // tables read in place are checked here
-    nodeB[v] = sqrt(2.0 * Dv);
-    // divergence
-    const long long ve = (long long)e * m.n;
+    const int el = threadIdx.x / m.n, p = threadIdx.x - el * m.n;
+    const int e = blockIdx.x * epb + el;
+    const bool own = el < epb && e < m.E;
+    const int N = m.N, i = p % N, j = p / N;
+    const long long v = (long long)e * m.n + p;
+    if (own) {
+        const int kx = e % m.K[0], ky = e / m.K[0];
+        const double x = m.lo[0] + (kx + r.xi[i]) * m.h[0];
+        const double y = m.dim == 2 ? m.lo[1] + (ky + r.xi[j]) * m.h[1] : 0.0;
+        double ux, uy;
+        node_drift(fu, m, v, x, y, ux, uy);
+        su[0][threadIdx.x] = ux;
+        su[1][threadIdx.x] = uy;
+        nodeU[v] = ux;
+        if (m.dim == 2) nodeU[V + v] = uy;
+        const double Dv = node_diffusion(fD, v, x, y);
+        if (fD.err && !(Dv >= 0.0)) atomicOr(fD.err, 4);  // tables read in place are checked here
+        nodeB[v] = sqrt(2.0 * Dv);
+        if (phi) phi[v] = phi0_nodal ? phi0_nodal[v] : phi0_at(fphi, m, x, y);  // null: new fields between steps
+    }
+    __syncthreads();
+    if (!own) return;
+    const double *ux = su[0] + el * m.n, *uy = su[1] + el * m.n;
     double dx = 0.0, dy = 0.0;
     for (int l = 0; l < N; ++l) {
-        double uxl, uyl, dummy;
-        if (m.dim == 1) {
-            node_drift(fu, m, ve + l, m.lo[0] + (kx + gauss_node(l, N)) * m.h[0], 0.0, uxl, dummy);
-            dx += lagrange_deriv(N, l, gauss_node(i, N)) * uxl;
-        } else {
-            node_drift(fu, m, ve + j * N + l, m.lo[0] + (kx + gauss_node(l, N)) * m.h[0], y, uxl, dummy);
-            dx += lagrange_deriv(N, l, gauss_node(i, N)) * uxl;
-            node_drift(fu, m, ve + l * N + i, x, m.lo[1] + (ky + gauss_node(l, N)) * m.h[1], dummy, uyl);
-            dy += lagrange_deriv(N, l, gauss_node(j, N)) * uyl;
-        }
+        dx += r.diff[i * N + l] * ux[m.dim == 1 ? l : j * N + l];
+        if (m.dim == 2) dy += r.diff[j * N + l] * uy[l * N + i];
     }
     nodeDiv[v] = dx / m.h[0] + (m.dim == 2 ? dy / m.h[1] : 0.0);
-    if (!Q) return;  // coefficients only (new fields between steps)
-    const double phi = phi0_nodal ? phi0_nodal[v] : phi0_at(fphi, m, x, y);
-    for (int s = 0; s < M; ++s) store_state(Q, (long long)s * V + v, phi);
 }
 
 // Interface coefficients.  1D: interface f (left face of element f) at
 // x_f = lo + f h.  2D: for each element the N points of its low-x face
 // (normal drift u_x) and of its low-y face (u_y), at the Gauss-node positions.
-__global__ void init_faces_kernel(Mesh m, FieldDev fu, FieldDev fD, double *faceU, double *faceB)
+__global__ void init_faces_kernel(Mesh m, FieldDev fu, FieldDev fD, const double *ref, double *faceU, double *faceB)
 {
+    const RefTab r(ref, m.N);
     const int nf = m.dim == 1 ? m.E + 1 : m.E * m.N;  // 1D: interfaces 0..K (K: x = hi)
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nf) return;
     if (m.dim == 1) {
         const double xf = v == m.E ? m.hi[0] : m.lo[0] + v * m.h[0];  // v = E: the boundary x = hi
-        face_fields(fu, fD, m, 0, 0, v, 0, xf, 0.0, faceU[v], faceB[v]);
+        face_fields(fu, fD, m, r, 0, 0, v, 0, xf, 0.0, faceU[v], faceB[v]);
         return;
     }
     const int e = v / m.N, f = v % m.N;
     const int kx = e % m.K[0], ky = e / m.K[0];
-    const double xv = m.lo[0] + kx * m.h[0], yv = m.lo[1] + (ky + gauss_node(f, m.N)) * m.h[1];
-    face_fields(fu, fD, m, 0, ky, kx, f, xv, yv, faceU[v], faceB[v]);
-    const double xh = m.lo[0] + (kx + gauss_node(f, m.N)) * m.h[0], yh = m.lo[1] + ky * m.h[1];
-    face_fields(fu, fD, m, 1, kx, ky, f, xh, yh, faceU[nf + v], faceB[nf + v]);
+    const double xv = m.lo[0] + kx * m.h[0], yv = m.lo[1] + (ky + r.xi[f]) * m.h[1];
+    face_fields(fu, fD, m, r, 0, ky, kx, f, xv, yv, faceU[v], faceB[v]);
+    const double xh = m.lo[0] + (kx + r.xi[f]) * m.h[0], yh = m.lo[1] + ky * m.h[1];
+    face_fields(fu, fD, m, r, 1, kx, ky, f, xh, yh, faceU[nf + v], faceB[nf + v]);
 }
 
 cudaError_t launch_init_fields(const Mesh &m, const FieldDev &u, const FieldDev &D, const FieldDev &phi0,
-                               const double *phi0_nodal_dev, double *xi, double *nodeU, double *nodeB,
-                               double *nodeDiv, double *faceU, double *faceB, void *Q, int M,
-                               int state_is_double, cudaStream_t st)
+                               const double *phi0_nodal_dev, const double *ref, double *nodeU, double *nodeB,
+                               double *nodeDiv, double *faceU, double *faceB, double *phi, cudaStream_t st)
 {
-    const long long V = (long long)m.E * m.n;
-    const int tb = 128;
-    const unsigned nb = unsigned((V + tb - 1) / tb);
-    if (state_is_double)
-        init_nodes_kernel<double><<<nb, tb, 0, st>>>(m, u, D, phi0, phi0_nodal_dev, xi, nodeU, nodeB, nodeDiv,
-                                                     static_cast<double *>(Q), M);
-    else
-        init_nodes_kernel<float2><<<nb, tb, 0, st>>>(m, u, D, phi0, phi0_nodal_dev, xi, nodeU, nodeB, nodeDiv,
-                                                     static_cast<float2 *>(Q), M);
+    const int epb = std::max(1, kInitThreads / 2 / m.n);
+    init_nodes_kernel<<<unsigned((m.E + epb - 1) / epb), unsigned((epb * m.n + 31) & ~31), 0, st>>>(
+        m, u, D, phi0, phi0_nodal_dev, ref, nodeU, nodeB, nodeDiv, phi, epb);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int nf = m.dim == 1 ? m.E + 1 : m.E * m.N;
-    init_faces_kernel<<<(nf + tb - 1) / tb, tb, 0, st>>>(m, u, D, faceU, faceB);
+    const int nf = m.dim == 1 ? m.E + 1 : m.E * m.N, tb = 128;
+    init_faces_kernel<<<(nf + tb - 1) / tb, tb, 0, st>>>(m, u, D, ref, faceU, faceB);
     return cudaGetLastError();
 }
 
@@ -519,26 +547,28 @@ __global__ void __launch_bounds__(32 * kFinWarps)
 
 // 2D faces on the upper domain boundaries (used with Dirichlet boundaries):
 // x = hi at the Gauss nodes of each row, then y = hi at those of each column.
-__global__ void init_faces_hi_kernel(Mesh m, FieldDev fu, FieldDev fD, double *faceUhi, double *faceBhi)
+__global__ void init_faces_hi_kernel(Mesh m, FieldDev fu, FieldDev fD, const double *ref, double *faceUhi,
+                                     double *faceBhi)
 {
+    const RefTab r(ref, m.N);
     const int nx = m.K[1] * m.N, ny = m.K[0] * m.N;
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nx + ny) return;
     if (v < nx) {  // x = hi at the Gauss nodes of element row v / N
-        const double y = m.lo[1] + (v / m.N + gauss_node(v % m.N, m.N)) * m.h[1];
-        face_fields(fu, fD, m, 0, v / m.N, m.K[0], v % m.N, m.hi[0], y, faceUhi[v], faceBhi[v]);
+        const double y = m.lo[1] + (v / m.N + r.xi[v % m.N]) * m.h[1];
+        face_fields(fu, fD, m, r, 0, v / m.N, m.K[0], v % m.N, m.hi[0], y, faceUhi[v], faceBhi[v]);
     } else {  // y = hi at the Gauss nodes of element column w / N
         const int w = v - nx;
-        const double x = m.lo[0] + (w / m.N + gauss_node(w % m.N, m.N)) * m.h[0];
-        face_fields(fu, fD, m, 1, w / m.N, m.K[1], w % m.N, x, m.hi[1], faceUhi[v], faceBhi[v]);
+        const double x = m.lo[0] + (w / m.N + r.xi[w % m.N]) * m.h[0];
+        face_fields(fu, fD, m, r, 1, w / m.N, m.K[1], w % m.N, x, m.hi[1], faceUhi[v], faceBhi[v]);
     }
 }
 
-cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, double *faceUhi, double *faceBhi,
-                                 cudaStream_t st)
+cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, const double *ref,
+                                 double *faceUhi, double *faceBhi, cudaStream_t st)
 {
     const int total = (m.K[0] + m.K[1]) * m.N;
-    init_faces_hi_kernel<<<(total + 127) / 128, 128, 0, st>>>(m, u, D, faceUhi, faceBhi);
+    init_faces_hi_kernel<<<(total + 127) / 128, 128, 0, st>>>(m, u, D, ref, faceUhi, faceBhi);
     return cudaGetLastError();
 }
 
@@ -740,8 +770,8 @@ void node_tables2d(int N, const double *xi, double *tab)
 
 cudaError_t preload_setup()
 {
-    cudaError_t e = prepare_kernel(init_nodes_kernel<double>);
-    if (e == cudaSuccess) e = prepare_kernel(init_nodes_kernel<float2>);
+    cudaError_t e = prepare_kernel(init_nodes_kernel);
+    if (e == cudaSuccess) e = prepare_kernel(ref_tables_kernel);
     if (e == cudaSuccess) e = prepare_kernel(init_faces_kernel);
     if (e == cudaSuccess) e = prepare_kernel(wiener_kernel);
     if (e == cudaSuccess) e = prepare_kernel(wiener_batch_kernel);
