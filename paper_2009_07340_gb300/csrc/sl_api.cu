@@ -226,28 +226,23 @@ cudaError_t ensure_loaded()
 namespace {
 
 // The time-step bounds (Eq. 1d_timestep with the node gap, and with the edge
-// distance) from the current node coefficients (host copy; synchronises the
-// context's stream).
+// distance) from the current node coefficients (reduced on the device;
+// synchronises the context's stream).
 int refresh_bounds(sl_ctx *c)
 {
     const sl::Mesh &m = c->m;
     const int dim = m.dim, N = m.N;
     const long long V = (long long)m.E * m.n;
-    std::vector<double> hu(size_t(dim) * V), hb(V);
-    cudaError_t e = cudaMemcpyAsync(hu.data(), c->nodeU, hu.size() * sizeof(double), cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(hb.data(), c->nodeB, hb.size() * sizeof(double), cudaMemcpyDeviceToHost, c->st);
+    double top[3] = {0.0, 0.0, 0.0};  // max |u_x|, |u_y|, sqrt(2 D)
+    cudaError_t e = sl::launch_bounds(c->nodeU, c->nodeB, dim, V, c->bounds, c->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(top, c->bounds, sizeof(top), cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) return SL_ERR_CUDA;
     double best = INFINITY, best_edge = INFINITY;
     const double gap = host_min_gap(N), edge = host_edge_gap(N);
-    double bmax = 0.0;
-    for (double b : hb) bmax = std::max(bmax, b);
     for (int d = 0; d < dim; ++d) {
-        double umax = 0.0;
-        for (long long v = 0; v < V; ++v) umax = std::max(umax, std::fabs(hu[size_t(d) * V + v]));
-        best = std::min(best, step_bound(umax, bmax, gap * m.h[d]));
-        best_edge = std::min(best_edge, step_bound(umax, bmax, edge * m.h[d]));
+        best = std::min(best, step_bound(top[d], top[2], gap * m.h[d]));
+        best_edge = std::min(best_edge, step_bound(top[d], top[2], edge * m.h[d]));
     }
     c->dtmax = best;
     c->dtedge = best_edge;
@@ -320,6 +315,7 @@ void sl_free(sl_ctx *c)
     sl::ctx_free(c, c->faceBhi);
     sl::ctx_free(c, c->xi);
     sl::ctx_free(c, c->ref);
+    sl::ctx_free(c, c->bounds);
     sl::ctx_free(c, c->nodeU);
     sl::ctx_free(c, c->nodeB);
     sl::ctx_free(c, c->nodeDiv);
@@ -421,7 +417,8 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
     const int nf = dim == 1 ? m.E + 1 : 2 * m.E * N;  // 1D: interfaces 0..K
     c->mom_chunk = 64;
     const int nc = (M + c->mom_chunk - 1) / c->mom_chunk;
-    bool ok = dalloc(c, &c->xi, N) == cudaSuccess && dalloc(c, &c->ref, size_t(N) * N + 3 * N) == cudaSuccess && dalloc(c, &c->nodeU, size_t(dim) * V) == cudaSuccess &&
+    bool ok = dalloc(c, &c->xi, N) == cudaSuccess && dalloc(c, &c->ref, size_t(N) * N + 3 * N) == cudaSuccess &&
+              dalloc(c, &c->bounds, 3) == cudaSuccess && dalloc(c, &c->nodeU, size_t(dim) * V) == cudaSuccess &&
               dalloc(c, &c->nodeB, V) == cudaSuccess && dalloc(c, &c->nodeDiv, V) == cudaSuccess &&
               dalloc(c, &c->faceU, nf) == cudaSuccess && dalloc(c, &c->faceB, nf) == cudaSuccess &&
               sl::ctx_alloc(c, &c->Q, size_t(M) * ncomp * V * c->state_elem) == cudaSuccess &&

@@ -191,6 +191,8 @@ cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, i
 // 2D coefficients on the faces x = hi ([Ky][N], u_x) and y = hi ([Kx][N], u_y).
 cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, const double *ref,
                                  double *faceUhi, double *faceBhi, cudaStream_t st);
+// Largest |u_d| and sqrt(2 D) over the V nodes: out[0], out[1] (2D), out[2].
+cudaError_t launch_bounds(const double *nodeU, const double *nodeB, int dim, long long V, double *out, cudaStream_t st);
 // Every sample set to `mean` (Eq. re-seed).
 cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, cudaStream_t st);
 
@@ -244,6 +246,7 @@ struct sl_ctx {
     double dtedge = 0.0;  // the same with the first node's distance to the element face
     // device memory owned by the context
     double *ref = nullptr;  // reference tables of the order [N N + 3 N] (launch_ref_tables)
+    double *bounds = nullptr;  // [3] largest |u_x|, |u_y|, sqrt(2 D) (launch_bounds)
     double *xi = nullptr, *nodeU = nullptr, *nodeB = nullptr, *nodeDiv = nullptr;
     double *faceU = nullptr, *faceB = nullptr;
     void *Q = nullptr;
