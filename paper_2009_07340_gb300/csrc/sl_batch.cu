@@ -36,6 +36,7 @@ struct Class1D {
     std::vector<int> ids;
     int grid = 0;       // persistent CTAs
     int max_grid = 0;   // occupancy limit
+    int block = sl::kMaxThreads1D;  // threads per CTA
     size_t smem = 0;
     int *d_counter = nullptr;
 };
@@ -123,12 +124,12 @@ int ensure_capacity(sl_batch *b, int steps)
     return SL_OK;
 }
 
-sl::Step1DArgs args1d(const sl_ctx *c, int steps)
+sl::Step1DArgs args1d(const sl_ctx *c, int steps, int S)
 {
     sl::Step1DArgs a;
     a.K = c->m.K[0];
     a.M = c->M;
-    a.S = c->S;
+    a.S = S;
     a.C = c->C;
     a.T = c->T;
     a.nsteps = steps;
@@ -208,6 +209,9 @@ size_t smem_1d(int precision, int N, int S, int T)
     return sl::step1d_smem_bytes_fp32(N, S, T);
 }
 
+// Sample fields of instance c that a CTA of `block` threads holds.
+int fields_per_cta(const sl_ctx *c, int block) { return std::max(1, std::min(block / c->T, c->M)); }
+
 // Device argument tables of one multi-instance step of `steps` steps
 // (allocated and uploaded before any capture; owned through `keep`).
 struct StepTables {
@@ -229,8 +233,9 @@ int prepare_step(sl_batch *b, int steps, StepTables &t, std::vector<void *> &kee
         std::vector<sl::Step1DArgs> args;
         std::vector<int> prefix(1, 0);
         for (int id : k.ids) {
-            args.push_back(args1d(b->inst[id], steps));
-            prefix.push_back(prefix.back() + (b->inst[id]->M + b->inst[id]->S - 1) / b->inst[id]->S);
+            const int S = fields_per_cta(b->inst[id], k.block);
+            args.push_back(args1d(b->inst[id], steps, S));
+            prefix.push_back(prefix.back() + (b->inst[id]->M + S - 1) / S);
         }
         sl::Batch1DLaunch l;
         l.args = upload(args, keep);
@@ -239,6 +244,7 @@ int prepare_step(sl_batch *b, int steps, StepTables &t, std::vector<void *> &kee
         l.ninst = int(k.ids.size());
         l.counter = k.d_counter;
         l.grid = k.grid;
+        l.block = k.block;
         l.smem = k.smem;
         t.l1.push_back(l);
     }
@@ -317,7 +323,7 @@ int enqueue_step(sl_batch *b, int steps, const StepTables &t)
             e = launch_1d_class(b, b->c1[it.idx], t.l1[it.idx], st);
         } else if (it.kind == 0) {
             const int id = it.idx;
-            const sl::Step1DArgs a = args1d(b->inst[id], steps);
+            const sl::Step1DArgs a = args1d(b->inst[id], steps, b->inst[id]->S);
             if (b->precision == SL_FP64) e = sl::launch_step1d_fp64(a, b->inst[id]->m.N, st);
             else if (b->precision == SL_MIXED) e = sl::launch_step1d_mixed(a, b->inst[id]->m.N, st);
             else e = sl::launch_step1d_fp32(a, b->inst[id]->m.N, st);
@@ -441,13 +447,35 @@ int sl_batch_create(sl_batch **out, int count, const sl_instance *specs, const s
         }
     }
     for (Class1D &k : b->c1) {
-        for (int id : k.ids) k.smem = std::max(k.smem, smem_1d(b->precision, k.N, b->inst[id]->S, b->inst[id]->T));
+        // Threads per CTA of the class: the fewest warps on the most loaded SM
+        // when the CTAs of all its items are dealt out evenly (the rule of
+        // geometry1d over the class), of equal ones the largest.
+        int widest = 1;
+        for (int id : k.ids) widest = std::max(widest, b->inst[id]->T);
+        long long best = -1, items = 0;
+        for (int block = 64; block <= sl::kMaxThreads1D; block += 32) {
+            if (block < widest) continue;
+            long long n = 0;
+            for (int id : k.ids) {
+                const int S = fields_per_cta(b->inst[id], block);
+                n += (b->inst[id]->M + S - 1) / S;
+            }
+            const long long load = (n + b->nsm - 1) / b->nsm * (block / 32);
+            if (best < 0 || load <= best) {
+                best = load;
+                items = n;
+                k.block = block;
+            }
+        }
+        for (int id : k.ids)
+            k.smem = std::max(k.smem, smem_1d(b->precision, k.N, fields_per_cta(b->inst[id], k.block), b->inst[id]->T));
         if (cudaMalloc(&k.d_counter, sizeof(int)) != cudaSuccess) {
             sl_batch_free(b);
             return SL_ERR_OOM;
         }
-        k.max_grid = 2 * b->nsm;  // refined by sl_batch_tune
-        k.grid = b->nsm;
+        // as many CTAs as 256 threads per SM hold, at most one per item; refined by sl_batch_tune
+        k.max_grid = 2 * b->nsm;
+        k.grid = int(std::max<long long>(1, std::min<long long>(items, (long long)b->nsm * (sl::kMaxThreads1D / k.block))));
     }
     for (Class2D &k : b->c2) {
         for (int id : k.ids) k.groups += (long long)b->inst[id]->m.E * b->inst[id]->M;
@@ -569,9 +597,9 @@ int sl_batch_tune(sl_batch *b, int probe_steps, double *best_ms)
             if (r == SL_OK) cudaEventElapsedTime(&ms, e0, e1);
             return r == SL_OK ? ms : -1.f;
         };
-        // occupancy bound of the persistent kernel: at most 4 CTAs per SM
-        // (256 threads each), fewer when shared memory is the limit
-        per_sm = std::max(1, std::min(4, int((227 * 1024) / std::max<size_t>(k.smem + 1024, 1))));
+        // occupancy bound of the persistent kernel: at most 1024 threads per
+        // SM, fewer when shared memory is the limit
+        per_sm = std::max(1, std::min(1024 / k.block, int((227 * 1024) / std::max<size_t>(k.smem + 1024, 1))));
         k.max_grid = per_sm * b->nsm;
         int best = b->nsm;
         float best_t = 1e30f;

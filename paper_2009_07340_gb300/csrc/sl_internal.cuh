@@ -132,6 +132,7 @@ struct Batch1DLaunch {
     int ninst;
     int *counter;            // device work counter (reset by the launcher)
     int grid;                // persistent CTAs
+    int block;               // threads per CTA
     size_t smem;             // dynamic shared memory per CTA
 };
 cudaError_t launch_step1d_batch_fp64(const Batch1DLaunch &b, int N, cudaStream_t st);
@@ -159,6 +160,8 @@ cudaError_t launch_step2d_fp64(const Step2DArgs &a, int N, cudaStream_t st);
 cudaError_t launch_step2d_fp32(const Step2DArgs &a, int N, cudaStream_t st);
 // two fields per sample (Q [M][2][E][n], faces [M][2][E][4N]), N <= 8
 cudaError_t launch_step2d_c2(const Step2DArgs &a, int N, bool fp64, cudaStream_t st);
+// Launch geometry of the 1D step (fields per CTA, CTAs per field, thread slots per field in a CTA).
+void geometry1d(int K, int M, int nsm, int max_threads, int &S, int &C, int &T);
 // The context's advance coefficients for step size dt (once per step size and fields).
 cudaError_t ensure_coef(sl_ctx *c, double dt);
 // The 1D advance coefficients of step size dt (Step1DArgs::coef), FP64 or float.

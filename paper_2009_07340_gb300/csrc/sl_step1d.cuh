@@ -646,7 +646,7 @@ cudaError_t launch_sl1d_step_kernel_batch_n(const Batch1DLaunch &b, cudaStream_t
     auto kern = sl1d_step_kernel_batch<N, MODE>;
     cudaError_t e = cudaMemsetAsync(b.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    kern<<<b.grid, kMaxThreads1D, b.smem, st>>>(b.args, b.prefix, b.ninst, b.counter);
+    kern<<<b.grid, b.block, b.smem, st>>>(b.args, b.prefix, b.ninst, b.counter);
     return cudaGetLastError();
 }
 
