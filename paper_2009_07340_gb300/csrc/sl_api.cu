@@ -297,8 +297,9 @@ cudaError_t ensure_coef(sl_ctx *c, double dt)
     const bool fp64 = c->precision == SL_FP64;
     const cudaError_t e =
         c->m.dim == 1 ? launch_coef1d(c->m, c->nodeU, c->nodeB, c->nodeDiv, c->faceU, c->faceB, dt, fp64, c->coef, c->st)
-                      : launch_coef2d(c->nodeU, c->nodeB, c->nodeDiv, (long long)c->m.E * c->m.n, dt, 4.0 / c->m.h[0],
-                                      4.0 / c->m.h[1], fp64, c->coef, c->st);
+                      : launch_coef2d(c->nodeU, c->nodeB, c->nodeDiv, c->faceU, c->faceB, (long long)c->m.E * c->m.n,
+                                      2ll * c->m.E * c->m.N, dt, 4.0 / c->m.h[0], 4.0 / c->m.h[1], fp64, c->coef,
+                                      c->st);
     if (e == cudaSuccess) {
         c->coef_dt = dt;
         c->coef_version = c->fields_version;
@@ -463,7 +464,7 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
               dalloc(c, &c->psq, size_t(nc) * ncomp * V) == cudaSuccess &&
               dalloc(c, &c->mean_tmp, ncomp * V) == cudaSuccess && dalloc(c, &c->m2_tmp, ncomp * V) == cudaSuccess &&
               dalloc(c, &c->err, 1) == cudaSuccess &&
-              sl::ctx_alloc(c, &c->coef, (dim == 1 ? size_t(3) * V + 2 * (m.E + 1) : size_t(5) * V) *
+              sl::ctx_alloc(c, &c->coef, (dim == 1 ? size_t(3) * V + 2 * (m.E + 1) : size_t(5) * V + size_t(4) * m.E * N) *
                                              (precision == SL_FP64 ? 8 : 4)) == cudaSuccess &&
               (dim == 1 || (dalloc(c, &c->faceUhi, size_t(m.K[0] + m.K[1]) * N) == cudaSuccess &&
                             dalloc(c, &c->faceBhi, size_t(m.K[0] + m.K[1]) * N) == cudaSuccess));

@@ -101,7 +101,8 @@ struct Step2DArgs {
     unsigned *slot_mark = nullptr, *slot_list = nullptr, *slot_ctl = nullptr;
     int f64_factor = 0;  // host: the FP32 remap factors its capacitance matrix in FP64 (SL_MIXED)
     const void *coef;      // [5][E][n] in the kernel's precision: 4 u_x dt / hx, 4 u_y dt / hy,
-                           // 4 b / hx, 4 b / hy (b = sqrt(2 D)), dt du_j/dx_j (launch_coef2d)
+                           // 4 b / hx, 4 b / hy (b = sqrt(2 D)), dt du_j/dx_j, then [2][2 E N] u dt and
+                           // b at the low-x and low-y faces (launch_coef2d)
     const double *nodeU;   // [2][E][n]
     const double *nodeB;   // [E][n]
     const double *nodeDiv; // [E][n]
@@ -168,8 +169,9 @@ cudaError_t ensure_coef(sl_ctx *c, double dt);
 cudaError_t launch_coef1d(const Mesh &m, const double *nodeU, const double *nodeB, const double *nodeDiv,
                           const double *faceU, const double *faceB, double dt, bool fp64, void *out, cudaStream_t st);
 // The 2D advance coefficients of step size dt (Step2DArgs::coef), FP64 or float.
-cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double *nodeDiv, long long V, double dt,
-                          double s4x, double s4y, bool fp64, void *out, cudaStream_t st);
+cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double *nodeDiv, const double *faceU,
+                          const double *faceB, long long V, long long nf, double dt, double s4x, double s4y, bool fp64,
+                          void *out, cudaStream_t st);
 // Host-side node tables of a 2D order (Step2DArgs::tab) from the nodes xi[N].
 void node_tables2d(int N, const double *xi, double *tab);
 // Reference tables of order N (derivative matrix, face values, nodes) and the nodes alone.

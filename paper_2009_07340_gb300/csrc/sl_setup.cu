@@ -730,10 +730,15 @@ cudaError_t launch_moments(const void *Q, int state_is_double, int M, long long 
 // the kernel's own precision (FP64 arithmetic is 1/64 of the FP32 rate).
 template <typename R>
 __global__ void coef2d_kernel(const double *__restrict__ nodeU, const double *__restrict__ nodeB,
-                              const double *__restrict__ nodeDiv, long long V, double dt, double s4x, double s4y,
-                              R *__restrict__ out)
+                              const double *__restrict__ nodeDiv, const double *__restrict__ faceU,
+                              const double *__restrict__ faceB, long long V, long long nf, double dt, double s4x,
+                              double s4y, R *__restrict__ out)
 {
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < nf) {  // nf = 2 E N <= V
+        out[5 * V + v] = R(__dmul_rn(faceU[v], dt));
+        out[5 * V + nf + v] = R(faceB[v]);
+    }
     if (v >= V) return;
     const double b = nodeB[v];
     out[v] = R(__dmul_rn(__dmul_rn(nodeU[v], dt), s4x));
@@ -743,14 +748,15 @@ __global__ void coef2d_kernel(const double *__restrict__ nodeU, const double *__
     out[4 * V + v] = R(__dmul_rn(dt, nodeDiv[v]));
 }
 
-cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double *nodeDiv, long long V, double dt,
-                          double s4x, double s4y, bool fp64, void *out, cudaStream_t st)
+cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double *nodeDiv, const double *faceU,
+                          const double *faceB, long long V, long long nf, double dt, double s4x, double s4y, bool fp64,
+                          void *out, cudaStream_t st)
 {
     const unsigned grid = unsigned((V + 255) / 256);
     if (fp64)
-        coef2d_kernel<double><<<grid, 256, 0, st>>>(nodeU, nodeB, nodeDiv, V, dt, s4x, s4y, static_cast<double *>(out));
+        coef2d_kernel<double><<<grid, 256, 0, st>>>(nodeU, nodeB, nodeDiv, faceU, faceB, V, nf, dt, s4x, s4y, static_cast<double *>(out));
     else
-        coef2d_kernel<float><<<grid, 256, 0, st>>>(nodeU, nodeB, nodeDiv, V, dt, s4x, s4y, static_cast<float *>(out));
+        coef2d_kernel<float><<<grid, 256, 0, st>>>(nodeU, nodeB, nodeDiv, faceU, faceB, V, nf, dt, s4x, s4y, static_cast<float *>(out));
     return cudaGetLastError();
 }
 

@@ -3,7 +3,7 @@
 // path's Gram matrix and its elimination), N <= 8.  Batches and served
 // requests carry one field; these are the single-instance kernels.  The
 // FP64 kernels are compiled in sl_step2d_c2_fp64.cu.
-#include "sl_step2d.cuh"
+#include "sl_step2d_launch.cuh"
 
 namespace sl {
 cudaError_t launch_step2d_c2_fp64(const Step2DArgs &a, int N, cudaStream_t st);

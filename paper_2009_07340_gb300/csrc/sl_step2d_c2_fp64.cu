@@ -1,7 +1,7 @@
 // 2D FP64 step kernels for two fields per sample, N <= 8 (see
 // sl_step2d_c2.cu; a translation unit of their own so that the two
 // precisions compile in parallel).
-#include "sl_step2d.cuh"
+#include "sl_step2d_launch.cuh"
 
 namespace sl {
 cudaError_t launch_step2d_c2_fp64(const Step2DArgs &a, int N, cudaStream_t st)

@@ -1,7 +1,7 @@
 // 2D step kernels of the FP32 remap with float-pair state (see
 // sl_step2d.cuh), N <= 12.  Both FP32 modes run them; SL_MIXED differs only
-// in the remap's fast kernel, which factors the capacitance matrix in FP64
-// (MODE 3).  The orders are compiled in sl_step2d_fp32_nNN.cu.
+// in the remap's iterative kernel, which factors the capacitance matrix in
+// FP64.  The orders are compiled in sl_step2d_fp32_nNN.cu.
 #include "sl_internal.cuh"
 
 namespace sl {

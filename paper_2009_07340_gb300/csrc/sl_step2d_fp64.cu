@@ -2,7 +2,7 @@
 // to 64 doubles in one thread's registers, N = 9..11 split it over two or
 // four lanes (sl_step2d_fp64_nNN.cu).  N = 12 would need 228 KB of shared
 // memory per element-sample, above the per-CTA limit.
-#include "sl_step2d.cuh"
+#include "sl_step2d_launch.cuh"
 
 namespace sl {
 cudaError_t launch_step2d_fp64_n9(const Step2DArgs &a, cudaStream_t st);
