@@ -33,12 +33,13 @@
 // a named barrier, row operands are loaded once for both nodes, and the
 // thread's row of C^{-1} stays in registers.  With one thread per node, two
 // warps and a named barrier per stage at N = 8, the kernel waited on barriers
-// and shared memory (43 % of the issue slots used).  Measured, with the FP32
-// preconditioner and this mapping against FP64 passes and that one: 64 x 64
-// elements, N = 8, FP32, two steps of 64 samples at half the node-gap step
-// 11.22 ms, now 8.22; 32 x 32, N = 6, FP64, one step of 32 samples 6.61 ms, now
-// 1.96; 32 x 32, N = 5, FP32, two steps of 64 samples with new fields 0.85 ms,
-// now 0.70; 19 x 23, N = 12, FP32, one step of 101 samples 2.97 ms, now 2.81.
+// and shared memory (43 % of the issue slots used; now 68 %, the shared-memory
+// pipe 78 % busy in phase 2).  Measured, with the FP32 preconditioner and this
+// mapping against FP64 passes and that one: 64 x 64 elements, N = 8, FP32, two
+// steps of 64 samples at half the node-gap step 11.37 ms, now 6.66; 32 x 32,
+// N = 6, FP64, one step of 32 samples 6.63 ms, now 1.89; 32 x 32, N = 5, FP32,
+// two steps of 64 samples with new fields 0.85 ms, now 0.68; 19 x 23, N = 12,
+// FP32, one step of 101 samples 2.97 ms, now 2.33.
 #pragma once
 #include "sl_step2d.cuh"
 
@@ -68,14 +69,9 @@ struct FGeo {
     static constexpr int RS = r4(N);     // rows [j][i] of a node field
     static constexpr int NR = odd4(N);   // rows read across lanes
     static constexpr int NTP = odd4(n);  // rows of the particles' basis values by node
-    // pivot block and threads per row of C's inversion
-    static constexpr int kCB = N == 8 || N == 9 ? 4 : 2;
-    static constexpr int kQB = N >= 11 ? 2 : 1;
-    static constexpr int CW = r4((F + kQB - 1) / kQB);  // columns per thread
-    static constexpr bool kRowsOneWarp = F * kQB <= 32;
-    static_assert(F * kQB <= TG && F % kCB == 0, "rows of C");
-    static constexpr int kGap = kQB > 1 ? 4 : 0;        // offset between column blocks of a published row
-    static constexpr int CR = r4(kQB * (CW + kGap));
+    static constexpr int kCB = 4;                       // pivot block of C's inversion
+    static constexpr bool kRowsOneWarp = F <= 32;
+    static constexpr int CR = odd4(F);                  // published pivot rows
     // per-group shared memory (floats)
     static constexpr int kW = N * NR;                   // one N x N table
     static constexpr int oW = 0;                        // Wx, Wx^T, Wy, Wy^T
@@ -84,14 +80,14 @@ struct FGeo {
     static constexpr int oRed = oDb + 2 * RS;           // [2][W][2] maxima
     static constexpr int oA = oRed + r4(4 * W);         // node field
     static constexpr int oB = oA + N * NR;              // node field, transposed rows
-    static constexpr int oVec = oB + N * NR;            // iterate, rows of RS
-    static constexpr int oRes = oVec + N * RS;          // residual: particles, then face points
-    static constexpr int oEnd1 = oRes + r4(n) + F;      // phase 1 ends here
+    static constexpr int oVec = oB + N * NR;            // iterate, rows of RS; a transposed field meanwhile
+    static constexpr int oRes = oVec + N * NR;          // residual: particles, then face points
+    // (at least the published rows of C's inversion, which these hold before the iteration)
+    static constexpr int oEnd1 = oRes + r4(n) + F > oA + 2 * kCB * CR ? oRes + r4(n) + F : oA + 2 * kCB * CR;
     static constexpr int oM = oEnd1;                    // Mx = Wx Wx^T, My
-    static constexpr int oU = oM + 2 * kW;              // hvx, hvy [4][N]; r / mu; u; M mu: [4N] each
-    static constexpr int oH = oU + 4 * F;               // hxT, hyT [N][NTP]
+    static constexpr int oU = oM + 2 * kW;              // hvx, hvy; r / mu; M mu ([4][RS] each); u [4N]
+    static constexpr int oH = oU + 12 * RS + F;         // hxT, hyT [N][NTP]
     static constexpr int oEnd2 = oH + 2 * N * NTP;
-    static_assert(2 * kCB * CR <= oEnd1 - oA, "published rows of C fit in the iteration's buffers");
     // FP64 buffers (doubles): the iterate; phase 2 also the particles' y basis
     // by node, their x basis times the residual ([N][NT64] each) and the face residuals
     static constexpr int NT64 = ((n + 1) / 2 | 1) * 2;  // rows an odd number of 16 bytes apart
@@ -133,8 +129,7 @@ __device__ __forceinline__ double rcp64(double x)
     return fma(y, fma(-x, y, 1.0), y);
 }
 
-// Rows of C^{-1} (creg: columns [col0, col0 + CW) of row `row`) from C's
-// structure, the factors in FP64 (the mixed form).  C = w^-2 I +
+// Row tig of C^{-1} (creg, threads tig < 4N) from C's structure, the factors in FP64 (the mixed form).  C = w^-2 I +
 // [[Gx (x) My, Cxy], [Cxy^T, Gy (x) Mx]] with Gx = [gx_s . gx_s'] (2 x 2), My =
 // Wy Wy^T and Cxy of rank 4 (its (s, s') blocks are hvy_s' hvx_s^T).  The
 // Kronecker blocks invert through the eigenvectors Q of Gx and Gy:
@@ -148,10 +143,10 @@ __device__ __forceinline__ double rcp64(double x)
 // GB300 runs FP64 at 2 lanes per clock per SM, so a warp-wide FP64 instruction
 // costs the same whatever its active lanes: the small FP64 steps spread their
 // work over the lanes of warp 0, and reciprocals are four FMA (rcp64).
-template <int N, int W, int TG, int NR, int RS, int CW>
+template <int N, int W, int TG, int NR, int RS>
 __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int wig, int bar_id, const float *gt,
-                                            const float *Mx, const float *My, const float *u4, float wi2, int row,
-                                            int col0, bool crow, float (&creg)[CW])
+                                            const float *Mx, const float *My, const float *u4, float wi2,
+                                            float (&creg)[4 * N])
 {
     constexpr int F = 4 * N;
     auto sync = [&]() {
@@ -165,7 +160,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
     float *A32 = reinterpret_cast<float *>(sm64 + 88);  // [4][N][N] Ainv in FP32
     float *Z32 = A32 + 4 * N * N;                       // [4N][4]: rows of Cxx^{-1} A, Cyy^{-1} B
     float *s32 = Z32 + 16 * N;                          // Qx [4], Qy [4], Mxx [16], M1 [16], Ti [16]
-    const float *hvx = u4, *hvy = u4 + 2 * N;  // hvx[s N + i] = (Wx gx_s)_i, hvy[s N + j] = (Wy gy_s)_j
+    const float *hvx = u4, *hvy = u4 + 2 * RS;  // hvx[s RS + i] = (Wx gx_s)_i, hvy[s RS + j] = (Wy gy_s)_j
     double *w64 = sm64 + 12;  // warp-0 scratch: [6] Gram entries, then [16] dots, [3][16] 4 x 4 matrices
     if (wig == 0) {  // the 2 x 2 eigen-decompositions (a Jacobi rotation each)
         if (lane < 6) {  // lane 3 d + e: d = 0 x, 1 y; e = 0: g0.g0, 1: g0.g1, 2: g1.g1
@@ -250,7 +245,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
     for (int e2 = tig; e2 < 8 * N; e2 += TG) {  // y and z, FP64
         const int v = e2 / N, k = e2 - v * N;
         const int mat = v < 4 ? v >> 1 : 2 + ((v - 4) >> 1);
-        const float *h = v < 4 ? hvy + (v & 1) * N : hvx + (v & 1) * N;
+        const float *h = v < 4 ? hvy + (v & 1) * RS : hvx + (v & 1) * RS;
         double acc = 0.0;
 #pragma unroll
         for (int k2 = 0; k2 < N; ++k2) acc = fma(Ainv[(mat * N + k) * N + k2], double(h[k2]), acc);
@@ -265,7 +260,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
         if (lane < 16) {
             const bool isz = lane >= 8;
             const int t = (lane >> 2) & 1, a1 = (lane >> 1) & 1, a2 = lane & 1;
-            const float *h = isz ? hvx + a1 * N : hvy + a1 * N;
+            const float *h = isz ? hvx + a1 * RS : hvy + a1 * RS;
             const double *v = yz + ((isz ? 4 : 0) + 2 * t + a2) * N;
             double acc = 0.0;
 #pragma unroll
@@ -336,10 +331,10 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             }
     }
     sync();
-    if (crow) {  // this thread's columns of row `row` of C^{-1}, assembled in FP32
-        const int s = (row / N) & 1, k = row % N;
-        const bool fx = row < 2 * N;
-        const float4 zr4 = *reinterpret_cast<const float4 *>(Z32 + 4 * row);
+    if (tig < F) {  // row tig of C^{-1}, assembled in FP32
+        const int s = (tig / N) & 1, k = tig % N;
+        const bool fx = tig < 2 * N;
+        const float4 zr4 = *reinterpret_cast<const float4 *>(Z32 + 4 * tig);
         const float zr[4] = {zr4.x, zr4.y, zr4.z, zr4.w};
         const float *Mxx = s32 + 8, *M1 = s32 + 24, *Tinv = s32 + 40;
         float rr[4], rp[4];  // the row's coefficients for its own block and the other
@@ -362,22 +357,19 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             for (int t = 0; t < 2; ++t) cq[s2][t] = Q32[2 * s + t] * Q32[2 * s2 + t];
         const float *Ab = A32 + (fx ? 0 : 2) * N * N + k * N;  // row k of the block's inverses t = 0, 1
 #pragma unroll
-        for (int jj = 0; jj < CW; ++jj) {
-            const int g2 = col0 + jj;
-            if (g2 < F) {
-                const int s2 = (g2 / N) & 1, k2 = g2 % N;
-                const bool same = fx == (g2 < 2 * N);
-                const float4 z2 = *reinterpret_cast<const float4 *>(Z32 + 4 * g2);
-                float v = (same ? rr[0] : rp[0]) * z2.x;
-                v = fmaf(same ? rr[1] : rp[1], z2.y, v);
-                v = fmaf(same ? rr[2] : rp[2], z2.z, v);
-                v = fmaf(same ? rr[3] : rp[3], z2.w, v);
-                if (same) {
-                    v = fmaf(s2 ? cq[1][0] : cq[0][0], Ab[k2], v);
-                    v = fmaf(s2 ? cq[1][1] : cq[0][1], Ab[N * N + k2], v);
-                }
-                creg[jj] = v;
+        for (int g2 = 0; g2 < F; ++g2) {
+            const int s2 = (g2 / N) & 1, k2 = g2 % N;
+            const bool same = fx == (g2 < 2 * N);
+            const float4 z2 = *reinterpret_cast<const float4 *>(Z32 + 4 * g2);
+            float v = (same ? rr[0] : rp[0]) * z2.x;
+            v = fmaf(same ? rr[1] : rp[1], z2.y, v);
+            v = fmaf(same ? rr[2] : rp[2], z2.z, v);
+            v = fmaf(same ? rr[3] : rp[3], z2.w, v);
+            if (same) {
+                v = fmaf(cq[s2][0], Ab[k2], v);
+                v = fmaf(cq[s2][1], Ab[N * N + k2], v);
             }
+            creg[g2] = v;
         }
     }
 }
@@ -750,15 +742,18 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
     };
 
     // conditioning of the tensor factors: ||Wx||_inf ||Wy||_inf against the
-    // largest tried.  FP32: in a model of 64 x 64 elements of N = 8 every case
-    // converged below these in the given iteration count (phase 2 stops
-    // converging first).  FP64 refines from a more modest start in phase 1, with
-    // all it meets up to half the node-gap step (35, 97, 186 and 361 at the most
-    // for N = 4, 6, 8 and 11 in a rotating drift), and further in phase 2, where
-    // its corrections only have to shrink.
-    constexpr float kCond = PHASE == 1 ? (kPair ? 512.0f : 25.0f * N) : (kPair ? 160.0f : 1024.0f);
-    constexpr int kIters = 8;
-    constexpr int kOuter = 10;  // FP64: corrections
+    // largest tried.  A direct solve costs a dozen whole iterations, so the FP32
+    // limits leave it to the iteration itself to give up, by its own progress:
+    // on 64 x 64 elements of N = 8 at half the node-gap step (64 samples) a limit
+    // of 160 in phase 2 sent 11.3 % of the groups to the direct solve (3.28 ms a
+    // step), 250 7.4 % (2.99), 400 6.8 % (3.03), 600 6.8 % (3.05).  FP64: phase 1
+    // refines to the end of the range; phase 2, with a normal-equation
+    // preconditioner of FP32, stops earlier; at N <= 4, where a direct solve is
+    // cheap, the ill-conditioned go there at once.
+    constexpr float kCond = kPair ? (PHASE == 1 ? 512.0f : 300.0f) : N <= 4 ? 100.0f : (PHASE == 1 ? 4096.0f : 1024.0f);
+    constexpr int kIters = kPair ? 16 : 8;
+    constexpr int kOuter = 24;  // FP64: corrections (ill-conditioned groups gain a digit or less in each)
+    constexpr float kShrink = 0.45f;  // and the slowest progress at which that many suffice
     bool done = false;
     {
         float sx = 0.f, sy = 0.f;
@@ -907,7 +902,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                             done = true;
                             break;
                         }
-                        if (o > 0 && !(d < 0.5f * before)) break;  // not converging
+                        if (o > 0 && !(d < kShrink * before)) break;  // not converging
                         before = d;
 #pragma unroll
                         for (int k = 0; k < NS; ++k)
@@ -948,11 +943,12 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
             }
         } else {
             float *Mx = gb + G::oM, *My = Mx + G::kW;
-            float *u4 = gb + G::oU, *mu4 = u4 + F, *uu4 = mu4 + F, *mm4 = uu4 + F;
+            float *u4 = gb + G::oU, *mu4 = u4 + 4 * RS, *mm4 = mu4 + 4 * RS, *uu4 = mm4 + 4 * RS;
+            const int fseg = tig / N * RS, fk = tig % N;  // face point tig: its side's row, its place there
             const float *hxT = gb + G::oH, *hyT = hxT + N * G::NTP;
             const float wb = float(a.w), wi2 = 1.f / (wb * wb);
             // products for C: Mx = Wx Wx^T, My = Wy Wy^T (kept for the iteration), and
-            // hvx[s][i] = sum_a Wx[i][a] gx_s[a] at u4[s N + i], hvy[s][j] = sum_b Wy[j][b] gy_s[b] at u4[(2 + s) N + j]
+            // hvx[s][i] = sum_a Wx[i][a] gx_s[a] at u4[s RS + i], hvy[s][j] = sum_b Wy[j][b] gy_s[b] at u4[(2 + s) RS + j]
 #pragma unroll
             for (int k = 0; k < NS; ++k)
                 if (on[k]) {
@@ -969,137 +965,123 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                 float p[N], q[N];
                 load_rowf<N>((s2 < 2 ? Wx : Wy) + k * NR, p);
                 load_rowf<N>(gt + s2 * RS, q);
-                u4[tig] = dotf<N>(p, q);
+                u4[fseg + fk] = dotf<N>(p, q);
             }
             sync();
-            constexpr int QB = G::kQB, CW = G::CW;
-            const bool crow = tig < F * QB;  // a thread holding (part of) a row of C^{-1}
-            const int row = tig / QB, col0 = (tig - row * QB) * CW;
-            float creg[CW];
-#pragma unroll
-            for (int jj = 0; jj < CW; ++jj) creg[jj] = 0.f;
+            float creg[F];  // thread tig < 4N: row tig of C, then of C^{-1}
             if constexpr (!FAC64) {
-                // C's rows are held by QB threads each (columns [col0, col0 + CW)),
-                // which assemble them from the 1D products and invert C in place
-                // (symmetric positive definite, eigenvalues >= w^-2).
-                if (crow) {
-                    const bool fx = row < 2 * N;
-                    const int s2 = (row / N) & 1, k = row % N;
-                    const float *g = gt + (row / N) * RS, *g0 = gt + (fx ? 0 : 2) * RS;
-                    float gg0 = 0.f, gg1 = 0.f;
+                // C's rows are held by a thread each, assembled from the 1D products
+                // and inverted in place (symmetric positive definite, eigenvalues >= w^-2).
+                const bool fx = tig < 2 * N;
+                const int s2 = (tig / N) & 1;
 #pragma unroll
-                    for (int m = 0; m < N; ++m) {
-                        gg0 = fmaf(g[m], g0[m], gg0);
-                        gg1 = fmaf(g[m], g0[RS + m], gg1);
-                    }
-                    const float *Mw = (fx ? My : Mx) + k * NR;  // Wy Wy^T along x faces, Wx Wx^T along y faces
+                for (int j = 0; j < F; ++j) creg[j] = 0.f;
+                if (tig < F) {
+                    float g[N], gv[N], gg0, gg1;
+                    load_rowf<N>(gt + fseg, g);
+                    load_rowf<N>(gt + (fx ? 0 : 2) * RS, gv);
+                    gg0 = dotf<N>(g, gv);
+                    load_rowf<N>(gt + (fx ? 1 : 3) * RS, gv);
+                    gg1 = dotf<N>(g, gv);
+                    float mw[N], h0[N];  // the row of M along this face; this side's hv
+                    load_rowf<N>((fx ? My : Mx) + fk * NR, mw);
+                    load_rowf<N>(u4 + (fx ? s2 : 2 + s2) * RS, h0);
+                    const float a0 = u4[(fx ? 2 : 0) * RS + fk], a1 = u4[(fx ? 3 : 1) * RS + fk];
 #pragma unroll
-                    for (int jj = 0; jj < CW; ++jj) {
-                        const int f2 = col0 + jj;
-                        if (QB == 1 || f2 < F) {
-                            const bool f2x = f2 < 2 * N;
-                            const int s3 = (f2 / N) & 1, k2 = f2 % N;
-                            float v;
-                            if (fx == f2x) v = (s3 == 0 ? gg0 : gg1) * Mw[k2];
-                            else if (fx) v = u4[(2 + s3) * N + k] * u4[s2 * N + k2];
-                            else v = u4[(2 + s2) * N + k2] * u4[s3 * N + k];
-                            creg[jj] = f2 == row ? v + wi2 : v;
-                        }
+                    for (int k2 = 0; k2 < N; ++k2) {
+                        const float d0 = gg0 * mw[k2], d1 = gg1 * mw[k2];  // sides 0, 1 of the same direction
+                        const float c0 = a0 * h0[k2], c1 = a1 * h0[k2];    // and of the other
+                        creg[k2] = fx ? d0 : c0;
+                        creg[N + k2] = fx ? d1 : c1;
+                        creg[2 * N + k2] = fx ? c0 : d0;
+                        creg[3 * N + k2] = fx ? c1 : d1;
                     }
+#pragma unroll
+                    for (int j = 0; j < F; ++j) creg[j] += j == tig ? wi2 : 0.f;
                 }
-                // Block Gauss-Jordan inversion in place with CB x CB pivot blocks
-                // (every pivot block of an SPD matrix is SPD: no pivoting).  Step K:
-                // the CB pivot rows publish themselves; after one barrier every
-                // thread inverts the pivot block P in registers and forms CB
-                // coefficients w: pivot row t takes row t of P^{-1}, any other row
-                // w = -C[r][K] P^{-1}; then C[r][j] <- C[r][j] + sum_m w_m C[K_m][j]
-                // outside the block (the pivot rows start from 0 instead of C[r][j])
-                // and C[r][K] <- w.  A thread reads its row's entries C[r][K] from
-                // the published rows: the partly inverted SPD matrix keeps
-                // C[r][k] = C[k][r] while r is not yet eliminated and
-                // C[r][k] = -C[k][r] once it is.  The published rows are
-                // double-buffered in the iteration's buffers.
+                // Block Gauss-Jordan inversion in place with 4 x 4 pivot blocks (every
+                // pivot block of an SPD matrix is SPD: no pivoting).  Step K: the pivot
+                // rows publish themselves; after one barrier every thread inverts the
+                // pivot block P in registers and forms the coefficients w: pivot row t
+                // takes row t of P^{-1}, any other row w = -C[r][K] P^{-1}; then
+                // C[r][j] <- C[r][j] + sum_m w_m C[K_m][j] outside the block (the pivot
+                // rows start from 0 instead of C[r][j]) and C[r][K] <- w.  The columns
+                // are rotated by a block in every step, so that the pivot block is
+                // always the first and one loop body serves all steps: unrolled, the
+                // steps overran the instruction cache (3.3 of 8.2 warps per issue
+                // waited for instructions at N = 8).
                 constexpr int CB = G::kCB, CR = G::CR;
-                auto pcol = [&](int j) { return j + (j / CW) * G::kGap; };  // column j's place in a published row
-                const int pcol0 = pcol(col0);
-                if (!G::kRowsOneWarp || wig == 0)  // uniform per warp; above one warp, every thread
+                if (!G::kRowsOneWarp || wig == 0) {  // uniform per warp; above one warp, every thread
+                    float *pb = fA;
+#pragma unroll 1
+                    for (int K = 0; K < F; K += CB) {
+                        const int t0 = tig - K;
+                        const bool pivot = t0 >= 0 && t0 < CB;
+                        if (pivot)
 #pragma unroll
-                for (int K = 0; K < F; K += CB) {
-                    float *pb = fA + ((K / CB) & 1) * CB * CR;
-                    const bool pivot = crow && row >= K && row < K + CB;
-                    if (pivot)
-#pragma unroll
-                        for (int jj = 0; jj < CW; jj += 4)
-                            *reinterpret_cast<float4 *>(pb + (row - K) * CR + pcol0 + jj) =
-                                make_float4(creg[jj], creg[jj + 1], creg[jj + 2], creg[jj + 3]);
-                    if constexpr (G::kRowsOneWarp) __syncwarp();
-                    else group_sync(bar_id, TG);
-                    if (crow) {
-                        float Pm[CB][CB];  // the pivot block, then its inverse
-#pragma unroll
-                        for (int t2 = 0; t2 < CB; ++t2)
-#pragma unroll
-                            for (int m = 0; m < CB; ++m) Pm[t2][m] = pb[t2 * CR + pcol(K) + m];
-#pragma unroll
-                        for (int p = 0; p < CB; ++p) {
-                            const float d = pdiv(1.f, Pm[p][p]);
-#pragma unroll
-                            for (int m = 0; m < CB; ++m) Pm[p][m] = m == p ? d : Pm[p][m] * d;
-#pragma unroll
-                            for (int q2 = 0; q2 < CB; ++q2)
-                                if (q2 != p) {
-                                    const float l = Pm[q2][p];
-#pragma unroll
-                                    for (int m = 0; m < CB; ++m)
-                                        Pm[q2][m] = m == p ? -l * d : fmaf(-l, Pm[p][m], Pm[q2][m]);
-                                }
-                        }
-                        const float sgn = row >= K ? 1.f : -1.f;
-                        float cr[CB], w[CB];
-#pragma unroll
-                        for (int t2 = 0; t2 < CB; ++t2) cr[t2] = -sgn * pb[t2 * CR + pcol(row)];
-#pragma unroll
-                        for (int m = 0; m < CB; ++m) {
-                            float other = 0.f, own = 0.f;
+                            for (int j = 0; j < F; j += 4)
+                                *reinterpret_cast<float4 *>(pb + t0 * CR + j) =
+                                    make_float4(creg[j], creg[j + 1], creg[j + 2], creg[j + 3]);
+                        if constexpr (G::kRowsOneWarp) __syncwarp();
+                        else group_sync(bar_id, TG);
+                        if (tig < F) {
+                            float Pm[CB][CB];  // the pivot block, then its inverse
 #pragma unroll
                             for (int t2 = 0; t2 < CB; ++t2) {
-                                other = fmaf(cr[t2], Pm[t2][m], other);
-                                own = row == K + t2 ? Pm[t2][m] : own;
+                                const float4 q = *reinterpret_cast<const float4 *>(pb + t2 * CR);
+                                Pm[t2][0] = q.x, Pm[t2][1] = q.y, Pm[t2][2] = q.z, Pm[t2][3] = q.w;
                             }
-                            w[m] = pivot ? own : other;
-                        }
 #pragma unroll
-                        for (int jj = 0; jj < CW; jj += 4) {
-                            float v[CB][4];
+                            for (int p = 0; p < CB; ++p) {
+                                const float d = pdiv(1.f, Pm[p][p]);
+#pragma unroll
+                                for (int m = 0; m < CB; ++m) Pm[p][m] = m == p ? d : Pm[p][m] * d;
+#pragma unroll
+                                for (int q2 = 0; q2 < CB; ++q2)
+                                    if (q2 != p) {
+                                        const float l = Pm[q2][p];
+#pragma unroll
+                                        for (int m = 0; m < CB; ++m)
+                                            Pm[q2][m] = m == p ? -l * d : fmaf(-l, Pm[p][m], Pm[q2][m]);
+                                    }
+                            }
+                            float w[CB];
 #pragma unroll
                             for (int m = 0; m < CB; ++m) {
-                                const float4 q = *reinterpret_cast<const float4 *>(pb + m * CR + pcol0 + jj);
-                                v[m][0] = q.x, v[m][1] = q.y, v[m][2] = q.z, v[m][3] = q.w;
+                                float other = 0.f, own = 0.f;
+#pragma unroll
+                                for (int t2 = 0; t2 < CB; ++t2) {
+                                    other = fmaf(-creg[t2], Pm[t2][m], other);
+                                    own = t0 == t2 ? Pm[t2][m] : own;
+                                }
+                                w[m] = pivot ? own : other;
                             }
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int j = col0 + jj + i;
-                                if (QB == 1 || j < F) {
-                                    if (j >= K && j < K + CB) {
-                                        float wj = w[0];
+                            for (int j = CB; j < F; j += 4) {
+                                float v[CB][4];
 #pragma unroll
-                                        for (int m = 1; m < CB; ++m) wj = j == K + m ? w[m] : wj;
-                                        creg[jj + i] = wj;
-                                    } else {
-                                        float acc = pivot ? 0.f : creg[jj + i];
+                                for (int m = 0; m < CB; ++m) {
+                                    const float4 q = *reinterpret_cast<const float4 *>(pb + m * CR + j);
+                                    v[m][0] = q.x, v[m][1] = q.y, v[m][2] = q.z, v[m][3] = q.w;
+                                }
 #pragma unroll
-                                        for (int m = 0; m < CB; ++m) acc = fmaf(w[m], v[m][i], acc);
-                                        creg[jj + i] = acc;
-                                    }
+                                for (int i = 0; i < 4; ++i) {
+                                    float acc = pivot ? 0.f : creg[j + i];
+#pragma unroll
+                                    for (int m = 0; m < CB; ++m) acc = fmaf(w[m], v[m][i], acc);
+                                    creg[j + i - CB] = acc;  // rotated
                                 }
                             }
+#pragma unroll
+                            for (int m = 0; m < CB; ++m) creg[F - CB + m] = w[m];
                         }
+                        pb = pb == fA ? fA + CB * CR : fA;
                     }
                 }
                 sync();  // the last step's published rows are read before the iteration overwrites them
             } else {
-                factor64_2d<N, W, TG, NR, RS, CW>(reinterpret_cast<double *>(gb + G::oEnd2), tig, lane, wig,
-                                              bar_id, gt, Mx, My, u4, wi2, row, col0, crow, creg);
+                factor64_2d<N, W, TG, NR, RS>(reinterpret_cast<double *>(gb + G::oEnd2), tig, lane, wig, bar_id, gt, Mx, My,
+                                              u4, wi2, creg);
             }
 
             // S^T res at the thread's nodes
@@ -1134,11 +1116,14 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                     z[k] = fmaf(wb, zf, z[k]);
                 }
             };
-            // d = G0^{-1} z at the thread's nodes
+            // d = G0^{-1} z at the thread's nodes (vec is overwritten)
             auto precondition = [&](const float (&z)[NS], float (&d)[NS]) {
 #pragma unroll
                 for (int k = 0; k < NS; ++k)
-                    if (on[k]) fA[jp[k] * RS + ip[k]] = z[k];
+                    if (on[k]) {
+                        fA[jp[k] * NR + ip[k]] = z[k];
+                        vec[ip[k] * NR + jp[k]] = z[k];
+                    }
                 sync();
                 // V0^{-T} z, first pass: [(j, a)] = sum_i Wx[i][a] z[(j, i)] (stored at [a][j]).
                 // With it, the face rows' u = E0 V0^{-T} z comes from z directly: since
@@ -1151,18 +1136,16 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                     for (int k = 0; k < NS; ++k) {
                         if (k == 0 || !kSameI) load_rowf<N>(WxT + ip[k] * NR, w);
                         float v[N];
-                        load_rowf<N>(fA + jp[k] * RS, v);
+                        load_rowf<N>(fA + jp[k] * NR, v);
                         const float tv = dotf<N>(w, v);
                         if (on[k]) fB[ip[k] * NR + jp[k]] = tv;
                     }
                 }
                 if (tig < F) {
-                    const int q = tig % N;
-                    const float *hv = u4 + (tig / N) * N;
-                    float rv = 0.f;
-#pragma unroll
-                    for (int m = 0; m < N; ++m) rv = fmaf(hv[m], tig < 2 * N ? fA[q * RS + m] : fA[m * RS + q], rv);
-                    mu4[tig] = rv;
+                    float h[N], v[N];
+                    load_rowf<N>(u4 + fseg, h);
+                    load_rowf<N>((tig < 2 * N ? fA : vec) + fk * NR, v);
+                    mu4[fseg + fk] = dotf<N>(h, v);
                 }
                 sync();
                 // second pass: t[(b, a)] = sum_j Wy[j][b] [(j, a)]; and u from r
@@ -1174,15 +1157,14 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         float w[N];
                         load_rowf<N>(WyT + jp[k] * NR, w);
                         const float tv = dotf<N>(w, v);
-                        if (on[k]) fA[jp[k] * RS + ip[k]] = tv;
+                        if (on[k]) fA[jp[k] * NR + ip[k]] = tv;
                     }
                 }
                 if (tig < F) {
-                    const float *Mm = (tig < 2 * N ? My : Mx) + (tig % N) * NR, *rv = mu4 + (tig / N) * N;
-                    float uv = 0.f;
-#pragma unroll
-                    for (int m = 0; m < N; ++m) uv = fmaf(Mm[m], rv[m], uv);
-                    uu4[tig] = uv;
+                    float m[N], v[N];
+                    load_rowf<N>((tig < 2 * N ? My : Mx) + fk * NR, m);
+                    load_rowf<N>(mu4 + fseg, v);
+                    uu4[tig] = dotf<N>(m, v);
                 }
                 sync();
                 // V0^{-1} t, first pass: [(b, i)] = sum_a Wx[i][a] t[(b, a)] (stored at [i][b]);
@@ -1193,36 +1175,30 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                     for (int k = 0; k < NS; ++k) {
                         if (k == 0 || !kSameI) load_rowf<N>(Wx + ip[k] * NR, w);
                         float v[N];
-                        load_rowf<N>(fA + jp[k] * RS, v);
+                        load_rowf<N>(fA + jp[k] * NR, v);
                         const float tv = dotf<N>(w, v);
                         if (on[k]) fB[ip[k] * NR + jp[k]] = tv;
                     }
                 }
-                if (!G::kRowsOneWarp || wig == 0) {
-                    float m = 0.f;
-                    if (crow) {
+                if (tig < F) {
+                    float m = 0.f, m2 = 0.f;
 #pragma unroll
-                        for (int jj = 0; jj < CW; jj += 4) {
-                            if (QB == 1 || col0 + jj < F) {  // 4N and CW are multiples of 4
-                                const float4 uv = *reinterpret_cast<const float4 *>(uu4 + col0 + jj);
-                                m = fmaf(creg[jj], uv.x, m);
-                                m = fmaf(creg[jj + 1], uv.y, m);
-                                m = fmaf(creg[jj + 2], uv.z, m);
-                                m = fmaf(creg[jj + 3], uv.w, m);
-                            }
-                        }
+                    for (int j = 0; j < F; j += 4) {
+                        const float4 uv = *reinterpret_cast<const float4 *>(uu4 + j);
+                        m = fmaf(creg[j], uv.x, m);
+                        m2 = fmaf(creg[j + 1], uv.y, m2);
+                        m = fmaf(creg[j + 2], uv.z, m);
+                        m2 = fmaf(creg[j + 3], uv.w, m2);
                     }
-                    if constexpr (QB == 2) m += __shfl_xor_sync(0xffffffffu, m, 1);
-                    if (crow && (QB == 1 || col0 == 0)) mu4[row] = m;  // r was last read in the previous stage
+                    mu4[fseg + fk] = m + m2;  // r was last read in the previous stage
                 }
                 sync();
                 // M mu: My mu_x,s and Mx mu_y,s
                 if (tig < F) {
-                    const float *Mm = (tig < 2 * N ? My : Mx) + (tig % N) * NR, *mv = mu4 + (tig / N) * N;
-                    float v = 0.f;
-#pragma unroll
-                    for (int m = 0; m < N; ++m) v = fmaf(Mm[m], mv[m], v);
-                    mm4[tig] = v;
+                    float m[N], v[N];
+                    load_rowf<N>((tig < 2 * N ? My : Mx) + fk * NR, m);
+                    load_rowf<N>(mu4 + fseg, v);
+                    mm4[fseg + fk] = dotf<N>(m, v);
                 }
                 sync();
                 // second pass, less V0^{-1} E0^T mu, which at node (i, j) is
@@ -1236,9 +1212,9 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         float w[N];
                         load_rowf<N>(Wy + j * NR, w);
                         float corr = mm4[j] * u4[i];
-                        corr = fmaf(mm4[N + j], u4[N + i], corr);
-                        corr = fmaf(u4[2 * N + j], mm4[2 * N + i], corr);
-                        corr = fmaf(u4[3 * N + j], mm4[3 * N + i], corr);
+                        corr = fmaf(mm4[RS + j], u4[RS + i], corr);
+                        corr = fmaf(u4[2 * RS + j], mm4[2 * RS + i], corr);
+                        corr = fmaf(u4[3 * RS + j], mm4[3 * RS + i], corr);
                         d[k] = dotf<N>(w, v) - corr;
                     }
                 }
@@ -1275,6 +1251,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                                 done = true;
                                 break;
                             }
+                            if (it > 3 && !(md < 0.75f * before)) break;  // not converging: left to the direct solve
                             before = md;
                         }
                         // stacked residual: particles phi* - V q, face points w (g - c) - w B q
@@ -1428,7 +1405,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                             done = true;
                             break;
                         }
-                        if (o > 1 && !(d < 0.5f * before)) break;  // not converging
+                        if (o > 1 && !(d < kShrink * before)) break;  // not converging
                         before = d;
                     }
                     if (cc + 1 < NCOMP) sync();
