@@ -69,3 +69,30 @@ def test_pdf_arguments(sl):
             with pytest.raises(sl.SLError) as e:
                 s.pdf(*bad)
             assert e.value.code == -1
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("B, lo, hi, M", [
+    (1, -1.0, 2.5, 300),               # one bin
+    (31, -1.0, 2.5, 4001),             # samples split over blocks, odd remainders
+    (383, 0.3, 0.7, 1600),             # the most bins that 32 values per block hold
+    (384, 0.3, 0.7, 1600),             # 16 values per block
+    (4096, -0.25, 0.5, 9000),          # two values per block, still split
+    (16, 1.0, 1.0 + 2.0 ** -20, 400),  # FP32 cannot tell the bins apart: the FP64 expression decides
+    (16, -1e31, 1e31, 400),            # beyond the FP32 path's range
+])
+def test_pdf_splits_and_edges(sl, orc, precision, B, lo, hi, M):
+    pb = I.config2(N=7, M=M, steps=0, K=5)  # 35 values: no multiple of a block's
+    rng = np.random.default_rng(B)
+    w = hi - lo
+    x = rng.uniform(lo - 0.1 * w, hi + 0.1 * w, size=(M, 35)).astype(np.float32).astype(np.float64)
+    edges = (lo + w / B * np.arange(B + 1)).astype(np.float32).astype(np.float64)
+    near = np.nextafter(edges.astype(np.float32), np.float32(np.inf)).astype(np.float64)
+    k = min(M, B + 1)
+    x[:k, 0], x[:k, 34] = edges[:k], near[:k]
+    x[:3, 1] = [np.inf, -np.inf, np.nan]
+    x = x.reshape(M, 5, 7)
+    with sl.Solver(pb, precision) as s:
+        s.set_samples(0, x)
+        got = s.pdf(B, lo, hi)
+    assert np.array_equal(got, orc.pdf(x, B, lo, hi))
