@@ -40,6 +40,11 @@
 // N = 6, FP64, one step of 32 samples 6.63 ms, now 1.89; 32 x 32, N = 5, FP32,
 // two steps of 64 samples with new fields 0.85 ms, now 0.68; 19 x 23, N = 12,
 // FP32, one step of 101 samples 2.97 ms, now 2.33.
+// Above N = 8 the 4N face points need more than one warp: two, with two nodes
+// per lane, up to N = 11 (a warp per 32 nodes, three or four, took 28.7, 35.1
+// and 44.0 ns per element-sample at N = 9, 10, 11 on 32 x 32 elements of 16
+// samples, now 25.1, 30.4 and 38.2), five at N = 12 (three nodes per lane in
+// two warps spill: 60.1 against 59.0 ns).
 #pragma once
 #include "sl_step2d.cuh"
 
@@ -51,7 +56,7 @@ struct FGeo {
     static constexpr bool kF64 = sizeof(R) == 8;
     // warps per group (FP64: one thread per node; its FP64 work is bound by
     // the FP64 pipe however it is dealt out)
-    static constexpr int W = kF64 ? (n + 31) / 32 : (N <= 8 ? 1 : N == 9 ? 3 : N <= 11 ? 4 : 5);
+    static constexpr int W = kF64 ? (n + 31) / 32 : (N <= 8 ? 1 : N <= 11 ? 2 : 5);
     static constexpr int TG = 32 * W;  // threads per group
     // lanes that hold nodes: whole rows of N where that needs no more slots, so
     // that a thread's nodes share their column i
@@ -87,7 +92,11 @@ struct FGeo {
     static constexpr int oM = oEnd1;                    // Mx = Wx Wx^T, My
     static constexpr int oU = oM + 2 * kW;              // hvx, hvy; r / mu; M mu ([4][RS] each); u [4N]
     static constexpr int oH = oU + 12 * RS + F;         // hxT, hyT [N][NTP]
-    static constexpr int oEnd2 = oH + 2 * N * NTP;
+    // rows of C^{-1}: in the thread's registers up to N = 8; above, FP32's two
+    // nodes per thread need those, and the rows are kept here
+    static constexpr bool kCShared = !kF64 && N > 8 && W == 2;
+    static constexpr int oC = oH + 2 * N * NTP;
+    static constexpr int oEnd2 = oC + (kCShared ? F * CR : 0);
     // FP64 buffers (doubles): the iterate; phase 2 also the particles' y basis
     // by node, their x basis times the residual ([N][NT64] each) and the face residuals
     static constexpr int NT64 = ((n + 1) / 2 | 1) * 2;  // rows an odd number of 16 bytes apart
@@ -118,13 +127,33 @@ __device__ __forceinline__ double scale2(double x, int k)
 {
     return x * __hiloint2double((min(max(k, -1022), 1023) + 1023) << 20, 0);
 }
-// 1 / x by two Newton-Raphson steps from the FP32 reciprocal (four FP64 FMA;
-// within an ulp), the division where the FP32 range does not hold x.
+// Conversions on the integer pipe (the conversion instructions run at the
+// FP64 rate): exact for normal floats and zero; to float rounded to nearest,
+// ties away, for values in its normal range.  Infinity and NaN become huge
+// numbers, subnormal floats wrong small ones: both only mislead the
+// preconditioner, whose iteration then fails and leaves the group to the
+// direct solve.
+__device__ __forceinline__ double wide(float x)
+{
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    return __hiloint2double(int((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), int(b << 29));
+}
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x));
+    const unsigned m = hi & 0x7fffffffu;
+    if (m < 0x38100000u || m >= 0x47e00000u) return m < 0x38100000u ? 0.f : float(x);
+    const unsigned v = ((m - 0x38000000u) << 3) + (lo >> 29) + ((lo >> 28) & 1u);
+    return __uint_as_float((hi & 0x80000000u) | v);
+}
+// 1 / x by two Newton-Raphson steps from the hardware's approximation (four
+// FP64 FMA); the division where that does not hold.
 __device__ __forceinline__ double rcp64(double x)
 {
-    const float f = float(x);
-    if (!(fabsf(f) > 1e-30f && fabsf(f) < 1e30f)) return 1.0 / x;
-    double y = double(__frcp_rn(f));
+    const unsigned m = unsigned(__double2hiint(x)) & 0x7fffffffu;
+    if (m < 0x20000000u || m > 0x5ff00000u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     y = fma(y, fma(-x, y, 1.0), y);
     return fma(y, fma(-x, y, 1.0), y);
 }
@@ -143,6 +172,9 @@ __device__ __forceinline__ double rcp64(double x)
 // GB300 runs FP64 at 2 lanes per clock per SM, so a warp-wide FP64 instruction
 // costs the same whatever its active lanes: the small FP64 steps spread their
 // work over the lanes of warp 0, and reciprocals are four FMA (rcp64).
+// Conversions run at the FP64 rate too and take the integer pipe instead:
+// with them and a reciprocal from a conversion the mixed form took 18.0, 28.9
+// and 78.1 ns per element-sample at N = 4, 8, 11, now 15.0, 23.6 and 64.3.
 template <int N, int W, int TG, int NR, int RS>
 __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int wig, int bar_id, const float *gt,
                                             const float *Mx, const float *My, const float *u4, float wi2,
@@ -168,7 +200,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             const float *ga = gt + (2 * d + (e == 2)) * RS, *gb = gt + (2 * d + (e != 0)) * RS;
             double acc = 0.0;
 #pragma unroll
-            for (int m = 0; m < N; ++m) acc = fma(double(ga[m]), double(gb[m]), acc);
+            for (int m = 0; m < N; ++m) acc = fma(wide(ga[m]), wide(gb[m]), acc);
             w64[lane] = acc;
         }
         __syncwarp();
@@ -191,10 +223,10 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             q[3] = cs;
             q[4] = l0;
             q[5] = l1;
-            s32[4 * d + 0] = float(cs);
-            s32[4 * d + 1] = float(sn);
-            s32[4 * d + 2] = float(-sn);
-            s32[4 * d + 3] = float(cs);
+            s32[4 * d + 0] = narrow(cs);
+            s32[4 * d + 1] = narrow(sn);
+            s32[4 * d + 2] = narrow(-sn);
+            s32[4 * d + 3] = narrow(cs);
         }
     }
     sync();
@@ -211,7 +243,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             const double lam = sm64[(mat >> 1) * 6 + 4 + (mat & 1)];
             const float *M = (mat < 2 ? My : Mx) + r * NR;  // My for the x faces, Mx for the y faces
 #pragma unroll
-            for (int j = 0; j < N; ++j) arow[j] = j == r ? fma(lam, double(M[j]), double(wi2)) : lam * double(M[j]);
+            for (int j = 0; j < N; ++j) arow[j] = j == r ? fma(lam, wide(M[j]), wide(wi2)) : lam * wide(M[j]);
         }
         if (kOneWarp ? wig == 0 : wig < 2) {  // uniform per warp
 #pragma unroll
@@ -238,7 +270,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 Ainv[(mat * N + r) * N + j] = arow[j];
-                A32[(mat * N + r) * N + j] = float(arow[j]);
+                A32[(mat * N + r) * N + j] = narrow(arow[j]);
             }
     }
     sync();
@@ -248,7 +280,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
         const float *h = v < 4 ? hvy + (v & 1) * RS : hvx + (v & 1) * RS;
         double acc = 0.0;
 #pragma unroll
-        for (int k2 = 0; k2 < N; ++k2) acc = fma(Ainv[(mat * N + k) * N + k2], double(h[k2]), acc);
+        for (int k2 = 0; k2 < N; ++k2) acc = fma(Ainv[(mat * N + k) * N + k2], wide(h[k2]), acc);
         yz[e2] = acc;
     }
     sync();
@@ -264,7 +296,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
             const double *v = yz + ((isz ? 4 : 0) + 2 * t + a2) * N;
             double acc = 0.0;
 #pragma unroll
-            for (int k = 0; k < N; ++k) acc = fma(double(h[k]), v[k], acc);
+            for (int k = 0; k < N; ++k) acc = fma(wide(h[k]), v[k], acc);
             dyz[lane] = acc;
         }
         __syncwarp();
@@ -308,9 +340,9 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
 #pragma unroll
         for (int m = 0; m < 4; ++m) mxx = fma(QT[4 * i4 + m], Qm[4 * m + j4], mxx);
         if (lane < 16) {
-            s32[8 + e] = float(mxx);                                // Mxx = Qm + Qm T^-1 Qm
-            s32[24 + e] = float((i4 == j4 ? 1.0 : 0.0) + QT[e]);    // M1 = I + Qm T^-1
-            s32[40 + e] = float(Pm[e]);                             // T^-1
+            s32[8 + e] = narrow(mxx);                                // Mxx = Qm + Qm T^-1 Qm
+            s32[24 + e] = narrow((i4 == j4 ? 1.0 : 0.0) + QT[e]);    // M1 = I + Qm T^-1
+            s32[40 + e] = narrow(Pm[e]);                             // T^-1
         }
     }
     if (tig < F) {  // row tig of Cxx^{-1} A (x faces) or Cyy^{-1} B (y faces)
@@ -327,7 +359,7 @@ __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int w
                     const double q = Qd[2 * s + t] * Qd[2 * (fx ? a1 : a2) + t];
                     acc = fma(q, yz[fx ? (2 * t + a2) * N + k : (4 + 2 * t + a1) * N + k], acc);
                 }
-                Z32[4 * f + 2 * a1 + a2] = float(acc);
+                Z32[4 * f + 2 * a1 + a2] = narrow(acc);
             }
     }
     sync();
@@ -1084,6 +1116,14 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                                               u4, wi2, creg);
             }
 
+            float *crow = gb + G::oC + (tig < F ? tig : 0) * G::CR;
+            if constexpr (G::kCShared) {
+                if (tig < F)
+#pragma unroll
+                    for (int j = 0; j < F; j += 4)
+                        *reinterpret_cast<float4 *>(crow + j) = make_float4(creg[j], creg[j + 1], creg[j + 2], creg[j + 3]);
+            }
+
             // S^T res at the thread's nodes
             auto transposed = [&](float (&z)[NS]) {
 #pragma unroll
@@ -1185,10 +1225,13 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
 #pragma unroll
                     for (int j = 0; j < F; j += 4) {
                         const float4 uv = *reinterpret_cast<const float4 *>(uu4 + j);
-                        m = fmaf(creg[j], uv.x, m);
-                        m2 = fmaf(creg[j + 1], uv.y, m2);
-                        m = fmaf(creg[j + 2], uv.z, m);
-                        m2 = fmaf(creg[j + 3], uv.w, m2);
+                        float4 cv;
+                        if constexpr (G::kCShared) cv = *reinterpret_cast<const float4 *>(crow + j);
+                        else cv = make_float4(creg[j], creg[j + 1], creg[j + 2], creg[j + 3]);
+                        m = fmaf(cv.x, uv.x, m);
+                        m2 = fmaf(cv.y, uv.y, m2);
+                        m = fmaf(cv.z, uv.z, m);
+                        m2 = fmaf(cv.w, uv.w, m2);
                     }
                     mu4[fseg + fk] = m + m2;  // r was last read in the previous stage
                 }
