@@ -8,8 +8,11 @@
 // carry two independent chains in one instruction, which halves the issue
 // slots of the O(N^2) parts:
 //   - advance / compositional update / state update: node pairs (2p, 2p+1);
-//   - barycentric weights: for each advected node j, the products over
-//     m-pairs of (Z_jm + delta_j - delta_m) (the m = j lane multiplies by 1);
+//   - barycentric weights: the differences of a node pair to each later node,
+//     each formed once and multiplied into both nodes' products (a third of
+//     the instructions of this part saved against every node's own product:
+//     30 steps of 501 sample fields of 777 elements at N = 11 in the mixed
+//     form 0.917 ms, now 0.833);
 //   - face bases: lane 0 = face xi = 0, lane 1 = face xi = 1;
 //   - remap: k outer over the advected nodes, pairs of Gauss nodes inner,
 //     with d'_ik = Z_ki + delta_k = -(zeta_i - zeta*_k); the recurrence on d'
@@ -157,22 +160,36 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
             ph[p] = fma2(sng[p * T + kl], Qh[p], dq);
         }
 
-        // barycentric weights w_j = 1 / prod_{m != j}(Z_jm + delta_j - delta_m)
+        // barycentric weights w_j = 1 / prod_{m != j}(Z_jm + delta_j - delta_m):
+        // every difference d of a node pair (2p, 2p + 1) to a later node m is
+        // formed once, for both products (the sign from m's side cancels in
+        // the pair)
         float w[N];
+        {
+            float2 up[NH];  // products over the later nodes
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            float zr[NP];
-            zrow(j, zr);
-            const float dj = lane_rt(dl[j >> 1], j & 1);
-            float2 acc = make_float2(1.f, 1.f);
+            for (int p = 0; p < NH; ++p) up[p] = make_float2(1.f, 1.f);
+#pragma unroll
+            for (int m = 0; m < N; ++m) {
+                const float2 nd = bc2(lane_rt(ndl[m >> 1], m & 1));
+                float2 acc = make_float2(1.f, 1.f);
+#pragma unroll
+                for (int p = 0; p < m / 2; ++p) {
+                    const float2 d = add2(make_float2(kTab.z[2 * p][m], kTab.z[2 * p + 1][m]), add2(dl[p], nd));
+                    up[p] = mul2(up[p], d);
+                    acc = p ? mul2(acc, d) : d;
+                }
+                w[m] = acc.x * acc.y;
+            }
 #pragma unroll
             for (int p = 0; p < NH; ++p) {
-                float2 d = add2(make_float2(zr[2 * p], zr[2 * p + 1]), add2(bc2(dj), ndl[p]));
-                if (2 * p == j) d.x = 1.f;
-                if (2 * p + 1 == j || 2 * p + 1 >= N) d.y = 1.f;
-                acc = mul2(acc, d);
+                w[2 * p] *= up[p].x;
+                if (2 * p + 1 < N) {
+                    const float d = kTab.z[2 * p][2 * p + 1] + (dl[p].x - dl[p].y);
+                    w[2 * p] *= d;
+                    w[2 * p + 1] *= -d * up[p].y;
+                }
             }
-            w[j] = acc.x * acc.y;
         }
         {
             float pp[N];
