@@ -182,14 +182,17 @@ cudaError_t launch_init_fields(const Mesh &m, const FieldDev &u, const FieldDev 
                                double *nodeDiv, double *faceU, double *faceB, double *phi, cudaStream_t st);
 cudaError_t launch_wiener(unsigned long long seed, long long step0, long long sample0, int nsteps, int M, int dim,
                           double sqrt_dt, double *out, cudaStream_t st);
+// err, err_out (both or neither): the second pass also copies *err to *err_out.
 cudaError_t launch_moments(const void *Q, int state_is_double, int M, long long V, int chunk,
-                           double *psum, double *psq, double *mean, double *m2, cudaStream_t st);
+                           double *psum, double *psq, double *mean, double *m2, cudaStream_t st,
+                           const int *err = nullptr, int *err_out = nullptr);
 // The first pass alone: per-chunk sums and sums of squares [ceil(M/chunk)][V].
 cudaError_t launch_moment_partials(const void *Q, int state_is_double, int M, long long V, int chunk,
                                    double *psum, double *psq, cudaStream_t st);
 // The second pass alone: chunk partials [nc][V] added in ascending c, / M.
 cudaError_t launch_moments_combine(const double *psum, const double *psq, int nc, long long V, long long M,
-                                   double *mean, double *m2, cudaStream_t st);
+                                   double *mean, double *m2, cudaStream_t st, const int *err = nullptr,
+                                   int *err_out = nullptr);
 // Per-node histogram of the samples into B bins over [lo, hi] (device [V][B]).
 cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, int B, double lo, double hi,
                        unsigned int *counts, cudaStream_t st);
@@ -258,7 +261,8 @@ struct sl_ctx {
     size_t state_elem = 8;
     double *dW = nullptr;
     int dW_cap = 0;  // steps the Wiener scratch holds
-    double *psum = nullptr, *psq = nullptr, *mean_tmp = nullptr, *m2_tmp = nullptr;
+    double *psum = nullptr, *psq = nullptr;
+    double *mean_tmp = nullptr;   // [2 vals + 1]: mean, second moment, error flags (sl_moments)
     int mom_chunk = 64;
     int *err = nullptr;
     void *faces2d = nullptr;  // 2D face-value scratch

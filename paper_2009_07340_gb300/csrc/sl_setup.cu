@@ -517,8 +517,10 @@ constexpr int kFinWarps = 8;
 
 __global__ void __launch_bounds__(32 * kFinWarps)
     moments_final_kernel(const double *__restrict__ psum, const double *__restrict__ psq, int nc, long long V,
-                         double M, double *__restrict__ mean, double *__restrict__ m2)
+                         double M, double *__restrict__ mean, double *__restrict__ m2, const int *__restrict__ err,
+                         int *__restrict__ err_out)
 {
+    if (err_out && blockIdx.x == 0 && threadIdx.x == 0) *err_out = *err;
     __shared__ double sa[kFinWarps][32], sb[kFinWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long v = (long long)blockIdx.x * 32 + lane;
@@ -791,18 +793,19 @@ cudaError_t launch_moment_partials(const void *Q, int state_is_double, int M, lo
 }
 
 cudaError_t launch_moments_combine(const double *psum, const double *psq, int nc, long long V, long long M,
-                                   double *mean, double *m2, cudaStream_t st)
+                                   double *mean, double *m2, cudaStream_t st, const int *err, int *err_out)
 {
-    moments_final_kernel<<<unsigned((V + 31) / 32), 32 * kFinWarps, 0, st>>>(psum, psq, nc, V, double(M), mean, m2);
+    moments_final_kernel<<<unsigned((V + 31) / 32), 32 * kFinWarps, 0, st>>>(psum, psq, nc, V, double(M), mean, m2, err,
+                                                                            err_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_moments(const void *Q, int state_is_double, int M, long long V, int chunk, double *psum,
-                           double *psq, double *mean, double *m2, cudaStream_t st)
+                           double *psq, double *mean, double *m2, cudaStream_t st, const int *err, int *err_out)
 {
     const int nc = (M + chunk - 1) / chunk;
     const cudaError_t e = launch_moment_partials(Q, state_is_double, M, V, chunk, psum, psq, st);
-    return e != cudaSuccess ? e : launch_moments_combine(psum, psq, nc, V, M, mean, m2, st);
+    return e != cudaSuccess ? e : launch_moments_combine(psum, psq, nc, V, M, mean, m2, st, err, err_out);
 }
 
 // Advance coefficients of the 2D step for step size dt, formed once per
