@@ -19,3 +19,15 @@ def orc():
 
     oracle.build()
     return oracle
+
+
+@pytest.fixture(autouse=True)
+def _collect_after_gpu_tests(request):
+    # the traceback that pytest.raises keeps holds the test's device tensors in
+    # a cycle; collected in a later test, they would change the allocator's
+    # figures while that test watches them
+    yield
+    if request.node.get_closest_marker("gpu"):
+        import gc
+
+        gc.collect()

@@ -212,3 +212,23 @@ def test_sample_ranges_shard_bitwise(sl):
         b.step()
         c.step()
         assert np.array_equal(np.concatenate([b.samples(), c.samples()]), whole)
+
+
+@pytest.mark.parametrize("K", [1, 3, 8, 32])
+@pytest.mark.parametrize("N", range(2, 17))
+def test_small_fp64_solves_equal_the_first_samples_of_large_ones(sl, N, K):
+    # a small FP64 solve deals an element's nodes out to lanes, a large one
+    # has a thread per element: the same operations in the same order.  Five
+    # samples (several fields in a block, the last one partly filled) against
+    # the first five of 20000 / K^(1/2); periodic, then Dirichlet with a weight.
+    pb = I.config2(N=N, M=5, steps=4, K=K)
+    pb["dt"] = 1e-6
+    large = I.with_(pb, M=int(20000 / K ** 0.5))
+    for extra in ({}, {"periodic": False, "bc_weight": 3.0,
+                       "ghost": np.stack([np.linspace(0.8, 1.2, 4), np.linspace(1.3, 0.9, 4)], axis=1)}):
+        got = []
+        for p in (I.with_(pb, **extra), I.with_(large, **extra)):
+            with sl.Solver(p, "fp64") as s:
+                s.step()
+                got.append(s.samples(0, 5))
+        assert np.array_equal(got[0], got[1])
