@@ -473,9 +473,10 @@ int sl_batch_create(sl_batch **out, int count, const sl_instance *specs, const s
             sl_batch_free(b);
             return SL_ERR_OOM;
         }
-        // as many CTAs as 256 threads per SM hold, at most one per item; refined by sl_batch_tune
+        // as many CTAs as 512 threads per SM hold (the FP32 kernels' register
+        // budget; FP64's wait for a slot), at most one per item; refined by sl_batch_tune
         k.max_grid = 2 * b->nsm;
-        k.grid = int(std::max<long long>(1, std::min<long long>(items, (long long)b->nsm * (sl::kMaxThreads1D / k.block))));
+        k.grid = int(std::max<long long>(1, std::min<long long>(items, (long long)b->nsm * (2 * sl::kMaxThreads1D / k.block))));
     }
     for (Class2D &k : b->c2) {
         for (int id : k.ids) k.groups += (long long)b->inst[id]->m.E * b->inst[id]->M;
