@@ -764,6 +764,19 @@ int sl_set_boundary(sl_ctx *c, int nsteps, const double *values)
     if (!c || nsteps < 0 || (nsteps > 0 && !values)) return SL_ERR_ARG;
     if (c->poisoned) return SL_ERR_STATE;
     if (c->periodic) return SL_ERR_ARG;
+    const void *src = values;
+    std::unique_ptr<float2[]> pairs;  // 1D FP32 modes: float pairs in the doubles' places
+    static_assert(sizeof(float2) == sizeof(double), "a pair in a double's place");
+    if (c->m.dim == 1 && c->precision != SL_FP64 && nsteps > 0) {
+        const size_t n = size_t(nsteps) * c->ghost_w;
+        pairs.reset(new (std::nothrow) float2[n]);
+        if (!pairs) return SL_ERR_OOM;
+        for (size_t i = 0; i < n; ++i) {
+            const float hi = float(values[i]);
+            pairs[i] = make_float2(hi, float(values[i] - double(hi)));
+        }
+        src = pairs.get();
+    }
     if (nsteps > c->ghost_cap) {
         sl::ctx_free(c, c->ghost);
         c->ghost = nullptr;
@@ -776,7 +789,7 @@ int sl_set_boundary(sl_ctx *c, int nsteps, const double *values)
         c->ghost_cap = nsteps;
     }
     if (nsteps > 0 &&
-        (cudaMemcpyAsync(c->ghost, values, size_t(nsteps) * c->ghost_w * sizeof(double), cudaMemcpyHostToDevice, c->st) !=
+        (cudaMemcpyAsync(c->ghost, src, size_t(nsteps) * c->ghost_w * sizeof(double), cudaMemcpyHostToDevice, c->st) !=
              cudaSuccess ||
          cudaStreamSynchronize(c->st) != cudaSuccess))
         return fail_cuda(c);

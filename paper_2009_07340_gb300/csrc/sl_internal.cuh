@@ -55,7 +55,8 @@ struct Step1DArgs {
     double inv_w2;         // 1 / w^2 of the boundary rows (0: hard constraints)
     int periodic;          // 0: Dirichlet boundaries with the ghost values below
     int ncomp;             // scalar fields per sample (1 or 2), state [M][ncomp][K][N]
-    const double *ghost;   // [nsteps][2] boundary values at x = lo, hi after each step (Dirichlet)
+    const double *ghost;   // [nsteps][2] boundary values at x = lo, hi after each step (Dirichlet); the FP32
+                           // modes: float pairs hi + lo in their place
     const double *xi;      // [N] reference nodes on [0,1]
     const void *coef;      // in the kernel's precision (launch_coef1d): [3][N][K] 4 u dt / h, 4 sqrt(2 D) / h
                            // and dt du/dx at the nodes, then [2][K + 1] u dt and sqrt(2 D) at the interfaces
