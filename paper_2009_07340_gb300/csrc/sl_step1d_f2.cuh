@@ -12,7 +12,7 @@
 //     each formed once and multiplied into both nodes' products (a third of
 //     the instructions of this part saved against every node's own product:
 //     30 steps of 501 sample fields of 777 elements at N = 11 in the mixed
-//     form 0.92 ms, now 0.86);
+//     form 0.917 ms, now 0.833);
 //   - face bases: lane 0 = face xi = 0, lane 1 = face xi = 1;
 //   - remap: k outer over the advected nodes, pairs of Gauss nodes inner,
 //     with d'_ik = Z_ki + delta_k = -(zeta_i - zeta*_k); the recurrence on d'
@@ -35,9 +35,7 @@ __device__ __forceinline__ float lane(const float2 *v)
 }
 __device__ __forceinline__ float lane_rt(const float2 &v, int odd) { return odd ? v.y : v.x; }
 
-// NCOMP fields per sample (state [M][NCOMP][K][N]) share all but the
-// compositional update, face values, jumps, mu and final evaluation.
-template <int N, int MODE, int NCOMP>
+template <int N, int MODE>
 __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int slot)
 {
     using Fac = typename Prec1D<MODE>::Fac;
@@ -48,8 +46,8 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int T = a.T, S = a.S, K = a.K;
-    float2 *sface = reinterpret_cast<float2 *>(smem_raw);                 // [2 buf][2 side][NCOMP][S][T] pairs
-    float2 *sal = sface + 4 * NCOMP * S * T;                                 // [NH][T] 4 u dt / h
+    float2 *sface = reinterpret_cast<float2 *>(smem_raw);                 // [2 buf][2 side][S][T] pairs
+    float2 *sal = sface + 4 * S * T;                                      // [NH][T] 4 u dt / h
     float2 *sbe = sal + NH * T;                                           // [NH][T] 4 b / h
     float2 *sng = sbe + NH * T;                                           // [NH][T] -dt du/dx
     float *sfa = reinterpret_cast<float *>(sng + NH * T);                 // [T + 1] u dt at interfaces
@@ -97,26 +95,23 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
     const bool active = sl < S && kl < Kc && s < a.M;
 
     float2 *Qg = reinterpret_cast<float2 *>(a.Q);
-    float2 Qh[NCOMP][NH], Ql[NCOMP][NH];  // state pairs: hi parts and lo parts of nodes (2p, 2p+1)
+    float2 Qh[NH], Ql[NH];  // state pairs: hi parts and lo parts of nodes (2p, 2p+1)
 #pragma unroll
-    for (int cc = 0; cc < NCOMP; ++cc) {
+    for (int p = 0; p < NH; ++p) {
+        Qh[p] = make_float2(0.f, 0.f);
+        Ql[p] = make_float2(0.f, 0.f);
+    }
+    if (active) {
+        const float2 *src = Qg + ((long long)s * K + (k0 + kl)) * N;
 #pragma unroll
-        for (int p = 0; p < NH; ++p) {
-            Qh[cc][p] = make_float2(0.f, 0.f);
-            Ql[cc][p] = make_float2(0.f, 0.f);
-        }
-        if (active) {
-            const float2 *src = Qg + (((long long)s * NCOMP + cc) * K + (k0 + kl)) * N;
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                const float2 v = src[j];
-                if (j & 1) {
-                    Qh[cc][j >> 1].y = v.x;
-                    Ql[cc][j >> 1].y = v.y;
-                } else {
-                    Qh[cc][j >> 1].x = v.x;
-                    Ql[cc][j >> 1].x = v.y;
-                }
+        for (int j = 0; j < N; ++j) {
+            const float2 v = src[j];
+            if (j & 1) {
+                Qh[j >> 1].y = v.x;
+                Ql[j >> 1].y = v.y;
+            } else {
+                Qh[j >> 1].x = v.x;
+                Ql[j >> 1].x = v.y;
             }
         }
     }
@@ -153,23 +148,16 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
         if (active && t + 1 < a.nsteps) dWn = a.dW[(long long)(t + 1) * a.M + s];
 
         // advance and compositional update, relative to c = Q_{N/2}
-        float ch[NCOMP], cl[NCOMP];
-        float2 dl[NH], ndl[NH], ph[NCOMP][NH];
+        const float ch = lane_rt(Qh[(N / 2) >> 1], (N / 2) & 1);
+        const float cl = lane_rt(Ql[(N / 2) >> 1], (N / 2) & 1);
+        float2 dl[NH], ndl[NH], ph[NH];
+        const float2 nch = bc2(-ch), ncl = bc2(-cl);
 #pragma unroll
         for (int p = 0; p < NH; ++p) {
             dl[p] = fma2(sbe[p * T + kl], bc2(dWr), sal[p * T + kl]);
             ndl[p] = mul2(dl[p], bc2(-1.f));
-        }
-#pragma unroll
-        for (int cc = 0; cc < NCOMP; ++cc) {
-            ch[cc] = lane_rt(Qh[cc][(N / 2) >> 1], (N / 2) & 1);
-            cl[cc] = lane_rt(Ql[cc][(N / 2) >> 1], (N / 2) & 1);
-            const float2 nch = bc2(-ch[cc]), ncl = bc2(-cl[cc]);
-#pragma unroll
-            for (int p = 0; p < NH; ++p) {
-                const float2 dq = add2(add2(Qh[cc][p], nch), add2(Ql[cc][p], ncl));
-                ph[cc][p] = fma2(sng[p * T + kl], Qh[cc][p], dq);
-            }
+            const float2 dq = add2(add2(Qh[p], nch), add2(Ql[p], ncl));
+            ph[p] = fma2(sng[p * T + kl], Qh[p], dq);
         }
 
         // barycentric weights w_j = 1 / prod_{m != j}(Z_jm + delta_j - delta_m):
@@ -220,6 +208,7 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
 
         // advected basis at both faces at once: E[j] = (E0_j, E1_j)
         float2 E[N];
+        float2 e = make_float2(0.f, 0.f);
         {
             float2 pre[N];
             pre[0] = make_float2(1.f, 1.f);
@@ -232,59 +221,49 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
                 E[j] = mul2(mul2(bc2(w[j]), pre[j]), suf);
                 if (j > 0) suf = mul2(suf, add2(Fp(j), bc2(lane_rt(ndl[j >> 1], j & 1))));
             }
-        }
-        float2 f0[NCOMP], f1[NCOMP];  // absolute face values as (hi, lo) pairs
 #pragma unroll
-        for (int cc = 0; cc < NCOMP; ++cc) {
-            float2 e = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < N; ++j) e = fma2(bc2(lane_rt(ph[cc][j >> 1], j & 1)), E[j], e);
-            two_sum(ch[cc], e.x, f0[cc].x, f0[cc].y);
-            f0[cc].y += cl[cc];
-            two_sum(ch[cc], e.y, f1[cc].x, f1[cc].y);
-            f1[cc].y += cl[cc];
+            for (int j = 0; j < N; ++j) e = fma2(bc2(lane_rt(ph[j >> 1], j & 1)), E[j], e);
         }
+        float2 f0, f1;  // absolute face values as (hi, lo) pairs
+        two_sum(ch, e.x, f0.x, f0.y);
+        f0.y += cl;
+        two_sum(ch, e.y, f1.x, f1.y);
+        f1.y += cl;
 
         const int buf = t & 1;
-        float2 *fL = sface + (buf * 2 + 0) * NCOMP * S * T;  // [NCOMP][S][T]
-        float2 *fR = sface + (buf * 2 + 1) * NCOMP * S * T;
+        float2 *fL = sface + (buf * 2 + 0) * S * T;
+        float2 *fR = sface + (buf * 2 + 1) * S * T;
         if (sl < S) {
-#pragma unroll
-            for (int cc = 0; cc < NCOMP; ++cc) {
-                fL[cc * S * T + sbase + kl] = f0[cc];
-                fR[cc * S * T + sbase + kl] = f1[cc];
-            }
+            fL[sbase + kl] = f0;
+            fR[sbase + kl] = f1;
         }
         if (C > 1)
             cluster.sync();
         else
             __syncthreads();
 
-        float2 gL[NCOMP], gR[NCOMP];
+        float2 gL, gR;
         {
             const float sigL = fmaf(sfb[kl], dWr, sfa[kl]);
             const float sigR = fmaf(sfb[kl + 1], dWr, sfa[kl + 1]);
-#pragma unroll
-            for (int cc = 0; cc < NCOMP; ++cc) {
-                float2 left_e1, right_e0;
-                if (C > 1) {
-                    left_e1 = *cluster.map_shared_rank(fR + cc * S * T + lnb_idx, lnb_rank);
-                    right_e0 = *cluster.map_shared_rank(fL + cc * S * T + rnb_idx, rnb_rank);
-                } else {
-                    left_e1 = fR[cc * S * T + sbase + lnb_idx];
-                    right_e0 = fL[cc * S * T + sbase + rnb_idx];
-                }
-                if (!a.periodic) {  // a domain boundary: the ghost value takes the missing neighbour's place
-                    if (k0 + kl == 0) left_e1 = ghost_face<float2>(a, 2 * t + 0);
-                    if (k0 + kl == K - 1) right_e0 = ghost_face<float2>(a, 2 * t + 1);
-                }
-                gL[cc] = sigL > 0.f ? left_e1 : f0[cc];
-                gR[cc] = sigR > 0.f ? f1[cc] : right_e0;
+            float2 left_e1, right_e0;
+            if (C > 1) {
+                left_e1 = *cluster.map_shared_rank(fR + lnb_idx, lnb_rank);
+                right_e0 = *cluster.map_shared_rank(fL + rnb_idx, rnb_rank);
+            } else {
+                left_e1 = fR[sbase + lnb_idx];
+                right_e0 = fL[sbase + rnb_idx];
             }
+            if (!a.periodic) {  // a domain boundary: the ghost value takes the missing neighbour's place
+                if (k0 + kl == 0) left_e1 = ghost_face<float2>(a, 2 * t + 0);
+                if (k0 + kl == K - 1) right_e0 = ghost_face<float2>(a, 2 * t + 1);
+            }
+            gL = sigL > 0.f ? left_e1 : f0;
+            gR = sigR > 0.f ? f1 : right_e0;
         }
 
         // 2x2 capacitance solve (I + E E^T) mu = E phi* - g
-        float mu0[NCOMP], mu1[NCOMP];
+        float mu0, mu1;
         {
             float2 gd = make_float2(0.f, 0.f);
             float g01 = 0.f;
@@ -295,38 +274,32 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
             }
             // I / w^2 + E E^T (w = 1 unless the caller weights the boundary rows)
             const Fac G00 = Fac(a.inv_w2) + Fac(gd.x), G01 = Fac(g01), G11 = Fac(a.inv_w2) + Fac(gd.y);
+            const Fac r0 = Fac((f0.x - gL.x) + (f0.y - gL.y));
+            const Fac r1 = Fac((f1.x - gR.x) + (f1.y - gR.y));
             const Fac det = G00 * G11 - G01 * G01;
             const Fac idet = Fac(1) / det;
-            bad |= !(det > Fac(0));
-#pragma unroll
-            for (int cc = 0; cc < NCOMP; ++cc) {
-                const Fac r0 = Fac((f0[cc].x - gL[cc].x) + (f0[cc].y - gL[cc].y));
-                const Fac r1 = Fac((f1[cc].x - gR[cc].x) + (f1[cc].y - gR[cc].y));
-                const Fac m0 = (G11 * r0 - G01 * r1) * idet;
-                const Fac m1 = (G00 * r1 - G01 * r0) * idet;
-                mu0[cc] = float(m0);
-                mu1[cc] = float(m1);
-                bad |= !isfinite(m0) || !isfinite(m1);
-            }
+            const Fac m0 = (G11 * r0 - G01 * r1) * idet;
+            const Fac m1 = (G00 * r1 - G01 * r0) * idet;
+            mu0 = float(m0);
+            mu1 = float(m1);
+            bad |= !(det > Fac(0)) || !isfinite(m0) || !isfinite(m1);
         }
 
-        // rw_j = (phi*_j - c - E0_j mu0 - E1_j mu1) w_j, and the remap to the
-        // Gauss nodes, pairs of nodes per instruction
-        float rw[NCOMP][N];
-        float2 A[NCOMP][NH], P[NH];
+        // rw_j = (phi*_j - c - E0_j mu0 - E1_j mu1) w_j
+        float rw[N];
 #pragma unroll
-        for (int cc = 0; cc < NCOMP; ++cc)
-#pragma unroll
-            for (int j = 0; j < N; ++j)
-                rw[cc][j] = (lane_rt(ph[cc][j >> 1], j & 1) - fmaf(E[j].x, mu0[cc], E[j].y * mu1[cc])) * w[j];
+        for (int j = 0; j < N; ++j)
+            rw[j] = (lane_rt(ph[j >> 1], j & 1) - fmaf(E[j].x, mu0, E[j].y * mu1)) * w[j];
+
+        // remap to the Gauss nodes, pairs of nodes per instruction
+        float2 A[NH], P[NH];
         {
             float zr[NP];
             zrow(0, zr);
             const float d0 = lane_rt(dl[0], 0);
 #pragma unroll
             for (int p = 0; p < NH; ++p) {
-#pragma unroll
-                for (int cc = 0; cc < NCOMP; ++cc) A[cc][p] = bc2(rw[cc][0]);
+                A[p] = bc2(rw[0]);
                 P[p] = add2(make_float2(zr[2 * p], zr[2 * p + 1]), bc2(d0));
             }
         }
@@ -335,40 +308,33 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
             float zr[NP];
             zrow(k, zr);
             const float2 dk = bc2(lane_rt(dl[k >> 1], k & 1));
+            const float2 rk = bc2(rw[k]);
 #pragma unroll
             for (int p = 0; p < NH; ++p) {
                 const float2 d = add2(make_float2(zr[2 * p], zr[2 * p + 1]), dk);
-#pragma unroll
-                for (int cc = 0; cc < NCOMP; ++cc) A[cc][p] = fma2(A[cc][p], d, mul2(bc2(rw[cc][k]), P[p]));
+                A[p] = fma2(A[p], d, mul2(rk, P[p]));
                 if (k + 1 < N) P[p] = mul2(P[p], d);
             }
         }
         // q = c + sign * A as an exact pair (TwoSum, two lanes per instruction)
 #pragma unroll
-        for (int cc = 0; cc < NCOMP; ++cc)
-#pragma unroll
-            for (int p = 0; p < NH; ++p) {
-                const float2 b = mul2(A[cc][p], bc2(kSign));
-                const float2 c = bc2(ch[cc]);
-                const float2 sm = add2(c, b);
-                const float2 bb = fma2(c, bc2(-1.f), sm);      // s - a
-                const float2 ta = fma2(bb, bc2(-1.f), sm);     // s - bb
-                const float2 ea = fma2(ta, bc2(-1.f), c);      // a - (s - bb)
-                const float2 eb = fma2(bb, bc2(-1.f), b);      // b - bb
-                Qh[cc][p] = sm;
-                Ql[cc][p] = add2(add2(ea, eb), bc2(cl[cc]));
-            }
+        for (int p = 0; p < NH; ++p) {
+            const float2 b = mul2(A[p], bc2(kSign));
+            const float2 sm = add2(bc2(ch), b);
+            const float2 bb = fma2(bc2(ch), bc2(-1.f), sm);          // s - a
+            const float2 ta = fma2(bb, bc2(-1.f), sm);               // s - bb
+            const float2 ea = fma2(ta, bc2(-1.f), bc2(ch));          // a - (s - bb)
+            const float2 eb = fma2(bb, bc2(-1.f), b);                // b - bb
+            Qh[p] = sm;
+            Ql[p] = add2(add2(ea, eb), bc2(cl));
+        }
     }
 
     if (active) {
+        float2 *dst = Qg + ((long long)s * K + (k0 + kl)) * N;
 #pragma unroll
-        for (int cc = 0; cc < NCOMP; ++cc) {
-            float2 *dst = Qg + (((long long)s * NCOMP + cc) * K + (k0 + kl)) * N;
-#pragma unroll
-            for (int j = 0; j < N; ++j)
-                dst[j] = (j & 1) ? make_float2(Qh[cc][j >> 1].y, Ql[cc][j >> 1].y)
-                                 : make_float2(Qh[cc][j >> 1].x, Ql[cc][j >> 1].x);
-        }
+        for (int j = 0; j < N; ++j)
+            dst[j] = (j & 1) ? make_float2(Qh[j >> 1].y, Ql[j >> 1].y) : make_float2(Qh[j >> 1].x, Ql[j >> 1].x);
         if (bad) atomicOr(a.err, 1);
     }
     if (C > 1) cluster.sync();
@@ -378,14 +344,7 @@ __device__ __forceinline__ void step1d_f2_body(const Step1DArgs &a, const int sl
 template <int N, int MODE>
 __global__ void __launch_bounds__(kMaxThreads1D, SL1D_FP32_MIN_BLOCKS) sl1d_step_kernel_f2(const Step1DArgs a)
 {
-    step1d_f2_body<N, MODE, 1>(a, int(blockIdx.x) / a.C);
-}
-
-// Two scalar fields per sample sharing the remap factorization.
-template <int N, int MODE>
-__global__ void __launch_bounds__(kMaxThreads1D, SL1D_FP32_MIN_BLOCKS) sl1d_step_kernel_f2_c2(const Step1DArgs a)
-{
-    step1d_f2_body<N, MODE, 2>(a, int(blockIdx.x) / a.C);
+    step1d_f2_body<N, MODE>(a, int(blockIdx.x) / a.C);
 }
 
 // Persistent batched launch over many instances of one order N (K <= 256,
@@ -411,26 +370,23 @@ __global__ void __launch_bounds__(kMaxThreads1D, SL1D_FP32_MIN_BLOCKS) sl1d_step
             else hi = mid - 1;
         }
         const Step1DArgs ai = args[lo];
-        step1d_f2_body<N, MODE, 1>(ai, item - item_prefix[lo]);
+        step1d_f2_body<N, MODE>(ai, item - item_prefix[lo]);
         __syncthreads();  // shared tables of this item are dead before the next fill
     }
 }
 
 template <int MODE>
-size_t step1d_f2_smem_bytes(int N, int S, int T, int ncomp = 1)
+size_t step1d_f2_smem_bytes(int N, int S, int T)
 {
     const int NE = N + (N & 1), NH = NE / 2;
-    return sizeof(float2) * (size_t(4) * ncomp * S * T + size_t(3) * NH * T) + sizeof(float) * 2 * (T + 1);
+    return sizeof(float2) * (size_t(4) * S * T + size_t(3) * NH * T) + sizeof(float) * 2 * (T + 1);
 }
 
 template <int N, int MODE>
 cudaError_t launch_step1d_f2_n(const Step1DArgs &a, cudaStream_t st)
 {
-    const size_t smem = step1d_f2_smem_bytes<MODE>(N, a.S, a.T, a.ncomp);
+    const size_t smem = step1d_f2_smem_bytes<MODE>(N, a.S, a.T);
     auto kern = sl1d_step_kernel_f2<N, MODE>;
-    if constexpr (MODE == SL_FP32) {
-        if (a.ncomp == 2) kern = sl1d_step_kernel_f2_c2<N, MODE>;  // (the mixed form has one field in 1D)
-    }
     cudaLaunchConfig_t cfg = {};
     const int slots = (a.M + a.S - 1) / a.S;
     cfg.gridDim = dim3(unsigned(slots * a.C));
@@ -451,8 +407,8 @@ template <int MODE>
 cudaError_t launch_step1d_f2_mode(const Step1DArgs &a, int N, cudaStream_t st)
 {
     switch (N) {
-    case 2: if constexpr (MODE == SL_MIXED) return launch_step1d_f2_n<2, MODE>(a, st); else return launch_step1d_n<2, MODE>(a, st);
-    case 3: if constexpr (MODE == SL_MIXED) return launch_step1d_f2_n<3, MODE>(a, st); else return launch_step1d_n<3, MODE>(a, st);
+    case 2: return launch_step1d_f2_n<2, MODE>(a, st);
+    case 3: return launch_step1d_f2_n<3, MODE>(a, st);
     case 4: return launch_step1d_f2_n<4, MODE>(a, st);
     case 5: return launch_step1d_f2_n<5, MODE>(a, st);
     case 6: return launch_step1d_f2_n<6, MODE>(a, st);
@@ -484,8 +440,8 @@ template <int MODE>
 cudaError_t launch_sl1d_step_kernel_f2_batch_mode(const Batch1DLaunch &b, int N, cudaStream_t st)
 {
     switch (N) {
-    case 2: if constexpr (MODE == SL_MIXED) return launch_sl1d_step_kernel_f2_batch_n<2, MODE>(b, st); else return launch_sl1d_step_kernel_batch_n<2, MODE>(b, st);
-    case 3: if constexpr (MODE == SL_MIXED) return launch_sl1d_step_kernel_f2_batch_n<3, MODE>(b, st); else return launch_sl1d_step_kernel_batch_n<3, MODE>(b, st);
+    case 2: return launch_sl1d_step_kernel_f2_batch_n<2, MODE>(b, st);
+    case 3: return launch_sl1d_step_kernel_f2_batch_n<3, MODE>(b, st);
     case 4: return launch_sl1d_step_kernel_f2_batch_n<4, MODE>(b, st);
     case 5: return launch_sl1d_step_kernel_f2_batch_n<5, MODE>(b, st);
     case 6: return launch_sl1d_step_kernel_f2_batch_n<6, MODE>(b, st);
@@ -503,17 +459,16 @@ cudaError_t launch_sl1d_step_kernel_f2_batch_mode(const Batch1DLaunch &b, int N,
     }
 }
 
-// Prepares the packed step kernels of one mode for the orders LO, LO + 1, ...
-template <int MODE, int LO, int... I>
+// Prepares the packed step kernels of one mode for every order.
+template <int MODE, int... I>
 cudaError_t preload_step1d_f2_seq(std::integer_sequence<int, I...>)
 {
     cudaError_t e = cudaSuccess;
     auto one = [&](auto f) {
         if (e == cudaSuccess) e = prepare_kernel(f);
     };
-    (one(sl1d_step_kernel_f2<I + LO, MODE>), ...);
-    if constexpr (MODE == SL_FP32) (one(sl1d_step_kernel_f2_c2<I + LO, MODE>), ...);
-    (one(sl1d_step_kernel_f2_batch<I + LO, MODE>), ...);
+    (one(sl1d_step_kernel_f2<I + 2, MODE>), ...);
+    (one(sl1d_step_kernel_f2_batch<I + 2, MODE>), ...);
     return e;
 }
 
