@@ -773,17 +773,21 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
         return int(m) - 5000;
     };
 
-    // conditioning of the tensor factors: ||Wx||_inf ||Wy||_inf against the
-    // largest tried.  A direct solve costs a dozen whole iterations, so the FP32
-    // limits leave it to the iteration itself to give up, by its own progress:
-    // on 64 x 64 elements of N = 8 at half the node-gap step (64 samples) a limit
-    // of 160 in phase 2 sent 11.3 % of the groups to the direct solve (3.28 ms a
-    // step), 250 7.4 % (2.99), 400 6.8 % (3.03), 600 6.8 % (3.05).  FP64: phase 1
-    // refines to the end of the range; phase 2, with a normal-equation
-    // preconditioner of FP32, stops earlier; at N <= 4, where a direct solve is
-    // cheap, the ill-conditioned go there at once.
-    constexpr float kCond = kPair ? (PHASE == 1 ? 512.0f : 300.0f) : N <= 4 ? 100.0f : (PHASE == 1 ? 4096.0f : 1024.0f);
-    constexpr int kIters = kPair ? 16 : 8;
+    // conditioning of the tensor factors, L = ||Wx||_inf ||Wy||_inf, against the
+    // largest tried.  FP32: the iteration contracts more slowly the larger L is,
+    // phase 2's (which squares the conditioning) first, and the line lies where
+    // what it accepts within kIters corrections is still as exact as the FP32
+    // residual.  On 64 x 64 elements of N = 8 at half the node-gap step with face
+    // jumps of 1e-3, one step is off from FP64 by (rms, relative to a group's own
+    // maximum) 2.4e-9 at L 16 to 64, 5.3e-8 at 64 to 128 and 3.6e-7 at 128 to 160;
+    // a limit of 300 with the rule below accepted groups of L 160 to 300 with
+    // 1.2e-5 (at most 2.3e-4), which the direct solve finishes to 2.5e-10.  That
+    // limit was 15 % faster there (2.80 against 3.29 ms a step of 64 samples).
+    // FP64: phase 1 refines to the end of the range; phase 2, with a normal-
+    // equation preconditioner of FP32, stops earlier; at N <= 4, where a direct
+    // solve is cheap, the ill-conditioned go there at once.
+    constexpr float kCond = kPair ? (PHASE == 1 ? 512.0f : 160.0f) : N <= 4 ? 100.0f : (PHASE == 1 ? 4096.0f : 1024.0f);
+    constexpr int kIters = 8;
     constexpr int kOuter = 24;  // FP64: corrections (ill-conditioned groups gain a digit or less in each)
     constexpr float kShrink = 0.45f;  // and the slowest progress at which that many suffice
     bool done = false;
@@ -804,13 +808,15 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
     }
 
     if (done) {
-        // Stopping of the FP32 iteration: the last correction below 1e-6 of
-        // max|x| + |c| (the remaining error is then that times the contraction
-        // rate), or the remaining error estimated from the last two corrections
-        // (d^2 / d_before) below 1e-7 of it.
-        auto settled = [&](float d, float before, float scale) {
-            return d < INFINITY && (d <= 1e-6f * scale || (before > 0.f && d < 0.5f * before && d * (d / before) <= 1e-7f * scale));
-        };
+        // Stopping of the FP32 iteration: the last correction d below 1e-6 of
+        // max|x| + |c|.  The remaining error is d rho / (1 - rho) at a contraction
+        // rate rho.  rho is not estimated from the corrections: the first ones are
+        // smooth, and their quotient promises a contraction that the worst-
+        // conditioned directions do not have.  Stopping on d^2 / d_before <= 1e-7 as
+        // well left one step of the groups of L 16 to 64 (see kCond) off by 1.6e-8
+        // rms instead of 2.4e-9, and the FP32 mean after 500 steps 1.8e-5 from FP64
+        // instead of 5.6e-6.
+        auto settled = [&](float d, float scale) { return d < INFINITY && d <= 1e-6f * scale; };
         // FP64: an FP32 correction is iterated to 1e-7 of itself (1e-8 estimated).
         // The outer iteration stops when the last correction is below 1e-13 of
         // max|x| + |c|, or when the remaining error estimated from the last two
@@ -874,7 +880,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                     sync();
                     float md;
                     maxima(md, mx);
-                    if (kPair ? settled(md, before, mx + scale0) : inner_settled(md, before, mx)) return true;
+                    if (kPair ? settled(md, mx + scale0) : inner_settled(md, before, mx)) return true;
                     // (FP64: a correction that stopped shrinking is left to the next residual)
                     if (!kPair && it > 0 && !(md < 0.5f * before)) return md < INFINITY;
                     before = md;
@@ -1290,7 +1296,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         if (it > 0) {
                             float md, mx;
                             maxima(md, mx);
-                            if (settled(md, before, mx + cref)) {
+                            if (settled(md, mx + cref)) {
                                 done = true;
                                 break;
                             }
@@ -1322,7 +1328,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         sync();
                         float md, mx;
                         maxima(md, mx);
-                        done = settled(md, before, mx + cref);
+                        done = settled(md, mx + cref);
                     }
                     if (cc + 1 < NCOMP) sync();
                 } else {
