@@ -783,10 +783,13 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
     // a limit of 300 with the rule below accepted groups of L 160 to 300 with
     // 1.2e-5 (at most 2.3e-4), which the direct solve finishes to 2.5e-10.  That
     // limit was 15 % faster there (2.80 against 3.29 ms a step of 64 samples).
-    // FP64: phase 1 refines to the end of the range; phase 2, with a normal-
-    // equation preconditioner of FP32, stops earlier; at N <= 4, where a direct
-    // solve is cheap, the ill-conditioned go there at once.
-    constexpr float kCond = kPair ? (PHASE == 1 ? 512.0f : 160.0f) : N <= 4 ? 100.0f : (PHASE == 1 ? 4096.0f : 1024.0f);
+    // FP64: phase 1 refines to the end of the range; phase 2's corrections are the
+    // FP32 iteration's and end where it does: with a limit of 1024, at the node-gap
+    // bound of 32 x 32 elements of N = 8, most of the groups between gave up (81815
+    // of all against 94509 now) and the others were up to 7e-13 off, where the
+    // direct solve leaves 3e-14; 266 against 282 ns per element-sample.  At N <= 4,
+    // where a direct solve is cheap, the ill-conditioned go there at once.
+    constexpr float kCond = !kPair && N <= 4 ? 100.0f : PHASE == 2 ? 160.0f : kPair ? 512.0f : 4096.0f;
     constexpr int kIters = 8;
     constexpr int kOuter = 24;  // FP64: corrections (ill-conditioned groups gain a digit or less in each)
     constexpr float kShrink = 0.45f;  // and the slowest progress at which that many suffice
@@ -817,18 +820,20 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
         // rms instead of 2.4e-9, and the FP32 mean after 500 steps 1.8e-5 from FP64
         // instead of 5.6e-6.
         auto settled = [&](float d, float scale) { return d < INFINITY && d <= 1e-6f * scale; };
-        // FP64: an FP32 correction is iterated to 1e-7 of itself (1e-8 estimated).
-        // The outer iteration stops when the last correction is below 1e-13 of
-        // max|x| + |c|, or when the remaining error estimated from the last two
-        // is below 1e-14 of it.  The first quotient is left out of the estimate:
-        // the first right-hand side is smooth, and the later ones, which are
-        // rounding errors, excite the worst-conditioned directions more.
+        // FP64: an FP32 correction is iterated to 1e-7 of itself (1e-8 estimated;
+        // what that leaves, the next residual shows).  The outer iteration stops
+        // when the last correction is below 1e-13 of max|x| + |c|; corrections
+        // shrink by kShrink or more, so that the remaining error is below it too.
+        // No estimate from two corrections here either: the directions that FP32
+        // resolves shrink by five digits a correction and hide the slow ones.
+        // With one (d^2 / d_before <= 1e-14), a step at the node-gap bound left
+        // groups of L 64 to 512 up to 1.6e-10 (N = 8) and 1e-8 (N = 10) from the
+        // solution.  Below that, where the third correction is rounding, both rules
+        // take three.
         auto inner_settled = [&](float d, float before, float scale) {
             return d < INFINITY && (d <= 1e-7f * scale || (before > 0.f && d < 0.5f * before && d * (d / before) <= 1e-8f * scale));
         };
-        auto refined = [&](int o, float d, float before, float scale) {
-            return d < INFINITY && (d <= 1e-13f * scale || (o > 1 && d < 0.5f * before && d * (d / before) <= 1e-14f * scale));
-        };
+        auto refined = [&](float d, float scale) { return d < INFINITY && d <= 1e-13f * scale; };
 
         if constexpr (PHASE == 1) {
             float wxr[NS][N], wyr[NS][N];  // the rows of Wx and Wy this thread applies
@@ -936,7 +941,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         maxima(mz, ms);
                         const float d = ldexpf(mx, max(top - e0, -140));
                         const float scale = ms + float(scale2(fabs(ch[cc]), -e0));
-                        if (refined(o, d, before, scale)) {
+                        if (refined(d, scale)) {
                             done = true;
                             break;
                         }
@@ -1450,7 +1455,7 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                         maxima(mz, ms);
                         const float d = ldexpf(dmax, max(top - e0, -140));
                         const float scale = ms + float(scale2(fabs(ch[cc]), -e0));
-                        if (o > 0 && refined(o, d, before, scale)) {
+                        if (o > 0 && refined(d, scale)) {
                             done = true;
                             break;
                         }

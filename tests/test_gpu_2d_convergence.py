@@ -1,8 +1,8 @@
-"""What the FP32 iteration of the 2D step accepts is as exact as its FP32
-residual, whatever the conditioning of a group's tensor factors: one step of
-rough states (face jumps of 1e-3) group by group against the FP64 kernels, by
-L = ||Wx||_inf ||Wy||_inf, and the moments after the whole horizon of the
-64 x 64 workload."""
+"""What the iterations of the 2D step accept is as exact as their residual,
+whatever the conditioning of a group's tensor factors: one step of rough
+states (face jumps of 1e-3) group by group, by L = ||Wx||_inf ||Wy||_inf, the
+FP32 forms against the FP64 kernels and those against the oracle; and the
+moments after the whole horizon of the 64 x 64 workload."""
 
 import numpy as np
 import pytest
@@ -59,6 +59,13 @@ def _conditioning(pb, dW):
     return np.array(out)
 
 
+def _rough_states(pb):
+    """[M][E][j][i]: 1 and a linear part per element, a jump at every face."""
+    N, E, xi = pb["N"], pb["K"][0] ** 2, _nodes(pb["N"])
+    c = 1e-3 * np.random.default_rng(N).uniform(-0.5, 0.5, size=(3, pb["M"], E, 1, 1))
+    return 1 + c[0] + c[1] * xi[None, :] + c[2] * xi[:, None]
+
+
 # Tolerances, relative to a group's own maximum.  An accepted group's error is
 # d rho / (1 - rho) with the last correction d <= 1e-6 of it.  Up to L = 64 the
 # contraction rate rho of the remap is at most 0.14 (a spectral radius that a
@@ -70,9 +77,7 @@ def _conditioning(pb, dW):
 @pytest.mark.parametrize("N,K,M", [(4, 64, 24), (6, 64, 12), (8, 64, 12), (10, 32, 16)])
 def test_accepted_groups_are_converged(sl, precision, N, K, M):
     pb = I.config3(M=M, steps=1, K=K, N=N, dt=1e-9)
-    xi, rng = _nodes(N), np.random.default_rng(N)
-    c = 1e-3 * rng.uniform(-0.5, 0.5, size=(3, M, K * K, 1, 1))
-    q0 = 1 + c[0] + c[1] * xi[None, :] + c[2] * xi[:, None]  # a jump at every face, [M][E][j][i]
+    q0 = _rough_states(pb)
     got = {}
     for prec in ("fp64", precision):
         with sl.Solver(pb, prec) as s:
@@ -91,6 +96,29 @@ def test_accepted_groups_are_converged(sl, precision, N, K, M):
     assert err[low].max() <= 2e-7
     assert mid.sum() == 0 or np.sqrt((err[mid] ** 2).mean()) <= 1e-6
     assert high.sum() == 0 or err[high].max() <= 2e-7
+
+
+# FP64: corrections shrink by 0.45 or more, the last is below 1e-13: 0.8e-13 of
+# the group remains in its faces and in its remap, which answers a face error
+# by a few times (its Lebesgue constant); rounding at a condition of L adds
+# L 2^-53 = 5e-13 at L = 4096.  1e-12 in all.
+@pytest.mark.parametrize("N", [4, 6, 8, 10])
+def test_fp64_groups_are_refined_to_the_end(sl, orc, N):
+    K, M = 16, 16
+    pb = I.config3(M=M, steps=1, K=K, N=N, dt=1e-9)
+    q0 = _rough_states(pb)
+    with sl.Solver(pb, "fp64") as s:
+        pb["dt"] = s.dt_max  # the whole node-gap bound: L over three orders of magnitude
+        s.set_samples(0, q0)
+        dW = s.wiener(0, 1, dt=pb["dt"])[0]
+        s.step(dt=pb["dt"], steps=1)
+        got = s.samples().reshape(M, K * K, N * N)
+        direct = s.fallbacks
+    ref = orc.run(pb, state_in=q0, want_states=True, nthreads=16, ns=M)["states"].reshape(got.shape)
+    L = _conditioning(pb, dW)
+    err = np.abs(got - ref).max(-1) / np.abs(ref).max(-1)
+    assert direct[1] < 0.5 * L.size  # most groups are the iteration's
+    assert err[L <= 4096].max() <= 1e-12
 
 
 def test_whole_horizon_of_the_64x64_workload(sl):
