@@ -237,9 +237,9 @@ __device__ __forceinline__ void step1d_body(const Step1DArgs &a, const int slot)
             const int i = idx / NP, m = idx - i * NP;
             sZ[idx] = m < N ? R(4.0 * (a.xi[i] - a.xi[m])) : R(0);
         }
-        if (threadIdx.x < N) {
-            sF0[threadIdx.x] = R(-4.0 * a.xi[threadIdx.x]);
-            sF1[threadIdx.x] = R(4.0 * (1.0 - a.xi[threadIdx.x]));
+        for (int m = threadIdx.x; m < N; m += blockDim.x) {  // a CTA of few elements has fewer threads than nodes
+            sF0[m] = R(-4.0 * a.xi[m]);
+            sF1[m] = R(4.0 * (1.0 - a.xi[m]));
         }
     }
 

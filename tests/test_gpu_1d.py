@@ -232,3 +232,13 @@ def test_small_fp64_solves_equal_the_first_samples_of_large_ones(sl, N, K):
                 s.step()
                 got.append(s.samples(0, 5))
         assert np.array_equal(got[0], got[1])
+
+
+def test_one_element_one_sample_of_two_nodes(sl, orc):
+    # FP64 N = 2: a block of one thread fills the node tables
+    pb = I.config2(N=2, M=1, steps=5, K=1)
+    pb["dt"] = 0.5 * orc.dt_max(pb)
+    ref = orc.run(pb, want_states=True, ns=1)["states"]
+    with sl.Solver(pb, "fp64") as s:
+        s.step()
+        assert np.abs(s.samples() - ref).max() / np.abs(ref).max() <= FP64_TOL

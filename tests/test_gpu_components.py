@@ -57,6 +57,20 @@ def test_two_components_equal_two_single_runs(sl, orc, precision, K, N, M):
         assert np.abs(st[:, 0] - ref).max() / np.abs(ref).max() <= FP64_TOL
 
 
+@pytest.mark.parametrize("K,N,M", [(3, 16, 4), (1, 16, 1), (2, 9, 2), (1, 3, 2), (15, 16, 1)])
+def test_two_components_with_fewer_threads_than_nodes(sl, orc, K, N, M):
+    # FP64: one thread per element and sample, so that K M < N threads fill the
+    # node tables of the block
+    pa, qa, qb = _pair_of_fields(orc, K, N, M, 5)
+    refs = [orc.run(pa, state_in=np.stack([q] * M), want_states=True, ns=M)["states"] for q in (qa, qb)]
+    with sl.Solver(I.with_(pa, components=2), "fp64") as s:
+        s.set_samples(0, np.stack([np.stack([qa, qb])] * M))
+        s.step()
+        st = s.samples()
+    for k in (0, 1):
+        assert np.abs(st[:, k] - refs[k]).max() / np.abs(refs[k]).max() <= FP64_TOL
+
+
 def _pair_of_fields_2d(orc, K, N, M, steps):
     pa = I.problem(2, K, (0.0, 0.0), (1.0, 1.0), N, M, steps, 0.0, 41, ("rotation", [2 * np.pi, 0.5, 0.5]),
                    ("sinsin", [0.004, 0.3, 2.0, 2.0]), ("gauss", [1.0, 0.15, 0.5, 0.6]))
