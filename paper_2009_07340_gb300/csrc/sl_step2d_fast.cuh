@@ -147,7 +147,8 @@ __device__ __forceinline__ float narrow(double x)
     return __uint_as_float((hi & 0x80000000u) | v);
 }
 // 1 / x by two Newton-Raphson steps from the hardware's approximation (four
-// FP64 FMA); the division where that does not hold.
+// FP64 FMA), within one unit in the last place of the quotient; the division
+// where the approximation's range ends.
 __device__ __forceinline__ double rcp64(double x)
 {
     const unsigned m = unsigned(__double2hiint(x)) & 0x7fffffffu;
