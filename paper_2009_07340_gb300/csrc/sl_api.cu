@@ -135,7 +135,7 @@ cudaError_t set_coefficients(sl_ctx *c, const sl_field *drift, const sl_field *d
         e = sl::launch_init_fields(m, du, dD, to_dev(phi0), phi0_nodal_dev, c->ref, c->nodeU, c->nodeB, c->nodeDiv,
                                    c->faceU, c->faceB, write_state ? c->mean_tmp : nullptr, c->st);
     if (e == cudaSuccess && write_state)  // every one of the [M][ncomp] fields of E n values
-        e = sl::launch_reseed(c->Q, c->precision == SL_FP64, c->M * c->ncomp, V, c->mean_tmp, c->st);
+        e = sl::launch_reseed(c->Q, c->precision == SL_FP64, c->M * c->ncomp, V, c->mean_tmp, c->nsm, c->st);
     if (e == cudaSuccess && m.dim == 2 && !c->periodic)  // read on Dirichlet boundaries only
         e = sl::launch_init_faces_hi(m, du, dD, c->ref, c->faceUhi, c->faceBhi, c->st);
     if (!device_tables) {
@@ -170,43 +170,6 @@ double step_bound(double umax, double bmax, double dx)
 }  // namespace
 
 namespace sl {
-
-// Launch geometry of the 1D step: C CTAs per sample field (a cluster above
-// max_threads elements), T thread slots per field in each, S fields per CTA.
-//
-// S: the step is bound by the arithmetic of the warps an SM is given, so the
-// rule takes the S that leaves the most loaded SM the fewest warps, counting
-// whole warps (a CTA of S K threads pads to one) and whole CTAs per SM; of
-// equal ones the largest (fewer coefficient tables).  A small solve spreads
-// over the SMs that way: 256 samples of 8 elements are 64 one-warp CTAs
-// instead of 8 of 256 threads (a whole solve of 100 FP64 steps at N = 6 2.65 ms,
-// now 1.30), and 10000 samples of 20 elements take 8 fields (160 threads, no
-// padding) instead of 12 (100 steps at N = 9 1.04 ms, now 1.00).
-// C: the fewest warps over the field's CTAs for the same reason; of equal
-// ones the smallest cluster.  777 elements take 5 CTAs of 156 slots
-// instead of 4 of 195 (30 steps of 501 fields, mixed, N = 11: 1.03 ms, now 0.92).
-void geometry1d(int K, int M, int nsm, int max_threads, int &S, int &C, int &T)
-{
-    auto warps = [](int threads) { return (threads + 31) / 32; };
-    C = (K + max_threads - 1) / max_threads;
-    if (C > 1) {
-        for (int c = C + 1; c <= kMaxCluster1D; ++c)
-            if (c * warps((K + c - 1) / c) < C * warps((K + C - 1) / C)) C = c;
-        T = (K + C - 1) / C;
-        S = 1;
-        return;
-    }
-    T = K;
-    S = 1;
-    long long best = -1;
-    for (int s = 1; s <= max_threads / K && s <= M; ++s) {
-        const long long ctas = (M + s - 1) / s, load = (ctas + nsm - 1) / nsm * warps(s * K);
-        if (best < 0 || load <= best) {
-            best = load;
-            S = s;
-        }
-    }
-}
 
 namespace {
 std::mutex g_load_mu;
@@ -272,7 +235,7 @@ int refresh_bounds(sl_ctx *c)
     const int dim = m.dim, N = m.N;
     const long long V = (long long)m.E * m.n;
     double top[3] = {0.0, 0.0, 0.0};  // max |u_x|, |u_y|, sqrt(2 D)
-    cudaError_t e = sl::launch_bounds(c->nodeU, c->nodeB, dim, V, c->bounds, c->st);
+    cudaError_t e = sl::launch_bounds(c->nodeU, c->nodeB, dim, V, c->bounds, c->nsm, c->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(top, c->bounds, sizeof(top), cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) return SL_ERR_CUDA;
@@ -416,6 +379,7 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
     sl_ctx *c = new (std::nothrow) sl_ctx;
     if (!c) return SL_ERR_OOM;
     cudaGetDevice(&c->device);
+    if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) c->nsm = 1;
     c->precision = precision;
     c->seed = opt ? opt->seed : 0ull;
     c->sample0 = opt ? opt->sample0 : 0ll;
@@ -521,9 +485,7 @@ int sl_init(sl_ctx **out, const sl_mesh *mesh, int N, int M, const sl_field *dri
     }
 
     if (dim == 1) {
-        int nsm = 0;
-        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) nsm = 1;
-        sl::geometry1d(m.K[0], M, nsm, sl::kMaxThreads1D, c->S, c->C, c->T);
+        sl::geometry1d(m.K[0], M, c->nsm, sl::kMaxThreads1D, c->S, c->C, c->T);
     }
     *out = c;
     return SL_OK;
@@ -673,6 +635,7 @@ int sl_step(sl_ctx *c, double dt, int steps)
             a.C = c->C;
             a.T = c->T;
             a.nsteps = n;
+            a.nsm = c->nsm;
             a.inv_w2 = c->inv_w2;
             a.periodic = c->periodic;
             a.ncomp = c->ncomp;
@@ -754,7 +717,7 @@ int sl_reseed(sl_ctx *c)
     const int dbl = c->precision == SL_FP64;
     if (sl::launch_moments(c->Q, dbl, c->M, V, c->mom_chunk, c->psum, c->psq, c->mean_tmp, nullptr, c->st) !=
             cudaSuccess ||
-        sl::launch_reseed(c->Q, dbl, c->M, V, c->mean_tmp, c->st) != cudaSuccess)
+        sl::launch_reseed(c->Q, dbl, c->M, V, c->mean_tmp, c->nsm, c->st) != cudaSuccess)
         return fail_cuda(c);
     return SL_OK;
 }
@@ -867,7 +830,7 @@ int sl_pdf_device(sl_ctx *c, int nbins, double lo, double hi, unsigned int *d_co
         return SL_ERR_ARG;
     if (c->poisoned) return SL_ERR_STATE;
     const long long V = c->vals;  // values per sample (components x nodes)
-    if (sl::launch_pdf(c->Q, c->precision == SL_FP64, c->M, V, nbins, lo, hi, d_counts, c->st) != cudaSuccess)
+    if (sl::launch_pdf(c->Q, c->precision == SL_FP64, c->M, V, nbins, lo, hi, d_counts, c->nsm, c->st) != cudaSuccess)
         return fail_cuda(c);
     return SL_OK;
 }

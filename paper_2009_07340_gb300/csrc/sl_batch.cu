@@ -133,6 +133,7 @@ sl::Step1DArgs args1d(const sl_ctx *c, int steps, int S)
     a.C = c->C;
     a.T = c->T;
     a.nsteps = steps;
+    a.nsm = c->nsm;
     a.inv_w2 = c->inv_w2;
     a.periodic = 1;  // batches hold periodic, single-field instances only
     a.ncomp = 1;

@@ -11,6 +11,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/sl.h"
+#include "sl_geometry1d.cuh"
 
 namespace sl {
 
@@ -25,8 +26,6 @@ struct TraceRange {
 };
 
 constexpr int kMaxN = 16;           // nodes per direction per element
-constexpr int kMaxThreads1D = 256;  // elements (threads) per CTA in the 1D kernel
-constexpr int kMaxCluster1D = 8;    // CTAs per sample field (portable cluster size)
 
 // Field descriptor copied to the device for the initialisation kernels.
 struct FieldDev {
@@ -52,6 +51,7 @@ struct Step1DArgs {
     int C;            // CTAs per sample field (cluster size)
     int T;            // thread slots per sample per CTA (>= elements per CTA)
     int nsteps;
+    int nsm;          // SMs of the device
     double inv_w2;         // 1 / w^2 of the boundary rows (0: hard constraints)
     int periodic;          // 0: Dirichlet boundaries with the ghost values below
     int ncomp;             // scalar fields per sample (1 or 2), state [M][ncomp][K][N]
@@ -162,8 +162,6 @@ cudaError_t launch_step2d_fp64(const Step2DArgs &a, int N, cudaStream_t st);
 cudaError_t launch_step2d_fp32(const Step2DArgs &a, int N, cudaStream_t st);
 // two fields per sample (Q [M][2][E][n], faces [M][2][E][4N]), N <= 8
 cudaError_t launch_step2d_c2(const Step2DArgs &a, int N, bool fp64, cudaStream_t st);
-// Launch geometry of the 1D step (fields per CTA, CTAs per field, thread slots per field in a CTA).
-void geometry1d(int K, int M, int nsm, int max_threads, int &S, int &C, int &T);
 // The context's advance coefficients for step size dt (once per step size and fields).
 cudaError_t ensure_coef(sl_ctx *c, double dt);
 // The 1D advance coefficients of step size dt (Step1DArgs::coef), FP64 or float.
@@ -196,14 +194,15 @@ cudaError_t launch_moments_combine(const double *psum, const double *psq, int nc
                                    int *err_out = nullptr);
 // Per-node histogram of the samples into B bins over [lo, hi] (device [V][B]).
 cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, int B, double lo, double hi,
-                       unsigned int *counts, cudaStream_t st);
+                       unsigned int *counts, int nsm, cudaStream_t st);
 // 2D coefficients on the faces x = hi ([Ky][N], u_x) and y = hi ([Kx][N], u_y).
 cudaError_t launch_init_faces_hi(const Mesh &m, const FieldDev &u, const FieldDev &D, const double *ref,
                                  double *faceUhi, double *faceBhi, cudaStream_t st);
 // Largest |u_d| and sqrt(2 D) over the V nodes: out[0], out[1] (2D), out[2].
-cudaError_t launch_bounds(const double *nodeU, const double *nodeB, int dim, long long V, double *out, cudaStream_t st);
+cudaError_t launch_bounds(const double *nodeU, const double *nodeB, int dim, long long V, double *out, int nsm,
+                          cudaStream_t st);
 // Every sample set to `mean` (Eq. re-seed).
-cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, cudaStream_t st);
+cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, int nsm, cudaStream_t st);
 
 // Module loading.  With lazy loading (the default), the first launch of a
 // kernel loads it, and a load may synchronise the whole device: a request
@@ -248,6 +247,7 @@ struct sl_ctx {
     long long sample0 = 0;
     cudaStream_t st = nullptr;
     int device = 0;
+    int nsm = 1;  // its SMs
     long long step = 0;
     int poisoned = 0;
     int bounds_stale = 0; // fields changed on the device: dtmax / dtedge recomputed when asked

@@ -668,7 +668,7 @@ static float pdf_eps(int B, double lo, double hi, double scale)
 }
 
 cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, int B, double lo, double hi,
-                       unsigned int *counts, cudaStream_t st)
+                       unsigned int *counts, int nsm, cudaStream_t st)
 {
     if (V == 0) return cudaSuccess;
     int lp = 5;  // 32 values of up to 383 bins, one of 4096: at most 48 KB
@@ -678,7 +678,7 @@ cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, i
     // about eight blocks per SM, each counting at least twice as many values
     // as its histogram has bins and a full unrolled pass
     const long long least = std::max<long long>(2LL * B, kPdfUnroll * (kPdfThreads >> lp));
-    const long long ny = std::max<long long>(1, std::min<long long>(M / least, (152LL * 8 + gx - 1) / gx));
+    const long long ny = std::max<long long>(1, std::min<long long>(M / least, (8LL * nsm + gx - 1) / gx));
     const int per = int((M + ny - 1) / ny);
     const dim3 grid{unsigned(gx), unsigned(M > 0 ? (M + per - 1) / per : 1)};
     const double scale = double(B) / (hi - lo);
@@ -718,14 +718,14 @@ __global__ void reseed_kernel(State *Q, const double *__restrict__ mean, int M, 
     for (long long s = blockIdx.y; s < M; s += gridDim.y) *reinterpret_cast<Vec *>(Q + s * V + v) = q;
 }
 
-cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, cudaStream_t st)
+cudaError_t launch_reseed(void *Q, int state_is_double, int M, long long V, const double *mean, int nsm, cudaStream_t st)
 {
     if (M == 0 || V == 0) return cudaSuccess;
     const bool two = V % 2 == 0 && reinterpret_cast<uintptr_t>(Q) % 16 == 0;
     const int tb = 128;
     const long long nx = (V / (two ? 2 : 1) + tb - 1) / tb;
     // about eight blocks of 128 threads per SM, each writing several samples' rows
-    const long long ny = std::max<long long>(1, std::min<long long>(std::min(M, 65535), (152LL * 8 + nx - 1) / nx));
+    const long long ny = std::max<long long>(1, std::min<long long>(std::min(M, 65535), (8LL * nsm + nx - 1) / nx));
     const dim3 grid{unsigned(nx), unsigned(ny)};
     if (state_is_double) {
         double *q = static_cast<double *>(Q);
@@ -761,11 +761,12 @@ __global__ void bounds_kernel(const double *__restrict__ nodeU, const double *__
     }
 }
 
-cudaError_t launch_bounds(const double *nodeU, const double *nodeB, int dim, long long V, double *out, cudaStream_t st)
+cudaError_t launch_bounds(const double *nodeU, const double *nodeB, int dim, long long V, double *out, int nsm,
+                          cudaStream_t st)
 {
     const cudaError_t e = cudaMemsetAsync(out, 0, 3 * sizeof(double), st);
     if (e != cudaSuccess) return e;
-    bounds_kernel<<<unsigned(std::min<long long>((V + 255) / 256, 152LL * 4)), 256, 0, st>>>(
+    bounds_kernel<<<unsigned(std::min<long long>((V + 255) / 256, 4LL * nsm)), 256, 0, st>>>(
         nodeU, nodeB, dim, V, reinterpret_cast<unsigned long long *>(out));
     return cudaGetLastError();
 }

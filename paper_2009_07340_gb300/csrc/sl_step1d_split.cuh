@@ -21,11 +21,9 @@
 
 namespace sl {
 
-constexpr int kSplitMaxThreads = 512;
-
 template <int N>
 struct Split1D {
-    static constexpr int G = N <= 8 ? 8 : 16;  // lanes per element (five at least: the chains)
+    static constexpr int G = split1d_lanes(N);  // lanes per element
     // per-element rows of G doubles: delta, F0 - delta, F1 - delta, raw weights,
     // their prefix products, pre0, suf0, pre1, suf1, phi*, E0, E1, r
     enum { DL, FA, FB, RAW, P0, S0, P1, S1, PP, PH, EA, EB, RW, ROWS };
@@ -180,33 +178,6 @@ __global__ void __launch_bounds__(kSplitMaxThreads) sl1d_split_kernel(const Step
     }
 }
 
-// Fields per CTA of the split kernel, 0 where the thread-per-element kernel is
-// the faster one: by the FP64 instructions per step of the most loaded SM,
-// where up to four warps (one per sub-partition) take the time of one.
-// At the line, 30 steps, thread per element and split: 31 elements of 150
-// samples at N = 6 353 and 234 us, at N = 16 1813 and 882; 8 of 1000 at N = 8
-// 555 and 477, at N = 16 1811 and 1536; on its other side 16 of 1000 take 610 us
-// at N = 8, one element per thread.
-inline int split1d_fields(const Step1DArgs &a, int N)
-{
-    const int G = N <= 8 ? 8 : 16;
-    if (a.ncomp != 1 || a.C != 1 || a.K * G > kSplitMaxThreads) return 0;
-    auto load = [](int S, int M, int threads) {
-        const long long ctas = (M + S - 1) / S, warps = (ctas + 151) / 152 * ((threads + 31) / 32);
-        return std::max(4ll, warps);
-    };
-    int best_S = 0;
-    long long best = (6ll * N * N + 22 * N) * load(a.S, a.M, a.S * a.T);
-    for (int S = 1; S * a.K * G <= kSplitMaxThreads && S <= a.M; ++S) {
-        const long long cost = (8ll * N + 60) * load(S, a.M, S * a.K * G);
-        if (cost < best) {
-            best = cost;
-            best_S = S;
-        }
-    }
-    return best_S;
-}
-
 template <int N>
 cudaError_t launch_split1d_n(Step1DArgs a, int S, cudaStream_t st)
 {
@@ -219,7 +190,6 @@ cudaError_t launch_split1d_n(Step1DArgs a, int S, cudaStream_t st)
 inline cudaError_t launch_split1d(const Step1DArgs &a, int N, int S, cudaStream_t st)
 {
     switch (N) {
-    case 2: return launch_split1d_n<2>(a, S, st);
     case 3: return launch_split1d_n<3>(a, S, st);
     case 4: return launch_split1d_n<4>(a, S, st);
     case 5: return launch_split1d_n<5>(a, S, st);
@@ -245,7 +215,7 @@ cudaError_t preload_split1d_seq(std::integer_sequence<int, I...>)
     auto one = [&](auto f) {
         if (e == cudaSuccess) e = prepare_kernel(f);
     };
-    (one(sl1d_split_kernel<I + 2>), ...);
+    (one(sl1d_split_kernel<I + 3>), ...);
     return e;
 }
 
