@@ -775,26 +775,25 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
     };
 
     // conditioning of the tensor factors, L = ||Wx||_inf ||Wy||_inf, against the
-    // largest tried.  FP32: the iteration contracts more slowly the larger L is,
-    // phase 2's (which squares the conditioning) first, and the line lies where
-    // what it accepts within kIters corrections is still as exact as the FP32
-    // residual.  On 64 x 64 elements of N = 8 at half the node-gap step with face
-    // jumps of 1e-3, one step is off from FP64 by (rms, relative to a group's own
-    // maximum) 2.4e-9 at L 16 to 64, 5.3e-8 at 64 to 128 and 3.6e-7 at 128 to 160;
-    // a limit of 300 with the rule below accepted groups of L 160 to 300 with
-    // 1.2e-5 (at most 2.3e-4), which the direct solve finishes to 2.5e-10.  That
-    // limit was 15 % faster there (2.80 against 3.29 ms a step of 64 samples).
-    // FP64: phase 1 refines to the end of the range; phase 2's corrections are the
-    // FP32 iteration's and end where it does: with a limit of 1024, at the node-gap
-    // bound of 32 x 32 elements of N = 8, most of the groups between gave up (81815
-    // of all against 94509 now) and the others were up to 7e-13 off, where the
-    // direct solve leaves 3e-14; 266 against 282 ns per element-sample.  At N <= 4,
-    // where a direct solve is cheap, the ill-conditioned go there at once.
-    constexpr float kCond = !kPair && N <= 4 ? 100.0f : PHASE == 2 ? 160.0f : kPair ? 512.0f : 4096.0f;
+    // largest tried: where what the iteration accepts within its corrections is as
+    // exact as its residual; above, the direct solve.  Phase 2 (which squares the
+    // conditioning) stops converging first, the mixed form's C^{-1}, rounded with
+    // its null directions (see below), before the others.  One step on 64 x 64
+    // elements of N = 8 at half the node-gap step with face jumps of 1e-3, off from
+    // FP64 relative to a group's own maximum: FP32 2.3e-9 rms (at most 1.7e-8) at L
+    // 64 to 160 and 6.3e-9 (6.7e-8) at 160 to 300; mixed 5.6e-7 (1.1e-5) at 128 to
+    // 160; the direct solve 2.5e-10.  A step of 64 samples takes 2.62 ms with the
+    // FP32 limit at 300, 3.25 at 160.  FP64, the whole node-gap step against the
+    // oracle: at most 3e-14 up to L = 512, 1.6e-13 at 512 to 1024 (the direct solve
+    // 3.4e-14).  At N <= 4, where a direct solve is cheap, FP64's ill-conditioned go
+    // there at once.
+    constexpr float kCond = kPair ? (PHASE == 1 ? 512.0f : FAC64 ? 160.0f : 300.0f)
+                                  : N <= 4 ? 100.0f : PHASE == 1 ? 4096.0f : 512.0f;
     constexpr int kIters = 8;
     constexpr int kOuter = 24;  // FP64: corrections (ill-conditioned groups gain a digit or less in each)
     constexpr float kShrink = 0.45f;  // and the slowest progress at which that many suffice
     bool done = false;
+    float cond = 0.f;
     {
         float sx = 0.f, sy = 0.f;
         if (tig < N) {
@@ -808,7 +807,8 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
         if constexpr (W > 1) sync();
         float mx, my;
         maxima(mx, my);
-        done = mx * my <= kCond;
+        cond = mx * my;
+        done = cond <= kCond;
     }
 
     if (done) {
@@ -1016,6 +1016,18 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
             if constexpr (!FAC64) {
                 // C's rows are held by a thread each, assembled from the 1D products
                 // and inverted in place (symmetric positive definite, eigenvalues >= w^-2).
+                // E0 E0^T has four null directions, one per corner: the corner's value
+                // along its x face is that along its y face, whatever the field.  There
+                // C is w^-2 alone, and an FP32 inverse of it as it stands loses digits in
+                // every direction.  u = E0 t has no part in them and E0^T takes none back,
+                // so that any multiple of them may be added to C: 4 L, the size of
+                // E0 E0^T (a model converged as well with the mean of its diagonal, less
+                // well with a tenth of it).  With it FP32 at L 128 to 160 is off by 2.2e-9
+                // rms where it was by 3.6e-7 (see kCond).  Groups left to the direct solve
+                // at N = 8, a tenth of the node-gap step, without and with it: w = 10 FP64
+                // 20 % and none, FP32 16 % and 0.4 %; w = 30 97 % and none, 84 % and 2 %
+                // (FP64 867 and 101 ns per element-sample).
+                const float kap = 4.f * cond;
                 const bool fx = tig < 2 * N;
                 const int s2 = (tig / N) & 1;
 #pragma unroll
@@ -1031,10 +1043,15 @@ __device__ __forceinline__ void sl2d_fast_group(const Step2DArgs &a0, const Step
                     load_rowf<N>((fx ? My : Mx) + fk * NR, mw);
                     load_rowf<N>(u4 + (fx ? s2 : 2 + s2) * RS, h0);
                     const float a0 = u4[(fx ? 2 : 0) * RS + fk], a1 = u4[(fx ? 3 : 1) * RS + fk];
+                    const float t0 = kap * fh0[fk], t1 = kap * fh1[fk];  // corner directions: entry fk of this face
+                    const float *hs = s2 ? fh1 : fh0;
 #pragma unroll
                     for (int k2 = 0; k2 < N; ++k2) {
-                        const float d0 = gg0 * mw[k2], d1 = gg1 * mw[k2];  // sides 0, 1 of the same direction
-                        const float c0 = a0 * h0[k2], c1 = a1 * h0[k2];    // and of the other
+                        float d0 = gg0 * mw[k2], d1 = gg1 * mw[k2];  // sides 0, 1 of the same direction
+                        const float v = fmaf(t0, fh0[k2], t1 * fh1[k2]);
+                        d0 += s2 ? 0.f : v;
+                        d1 += s2 ? v : 0.f;
+                        const float c0 = fmaf(-t0, hs[k2], a0 * h0[k2]), c1 = fmaf(-t1, hs[k2], a1 * h0[k2]);  // of the other
                         creg[k2] = fx ? d0 : c0;
                         creg[N + k2] = fx ? d1 : c1;
                         creg[2 * N + k2] = fx ? c0 : d0;

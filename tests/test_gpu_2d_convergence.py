@@ -70,9 +70,10 @@ def _rough_states(pb):
 # d rho / (1 - rho) with the last correction d <= 1e-6 of it.  Up to L = 64 the
 # contraction rate rho of the remap is at most 0.14 (a spectral radius that a
 # dense model of such elements gave at the whole node-gap step): 1.6e-7, and
-# 2.8e-8 for the faces (0.027); together 2e-7.  From 64 to 160 rho may reach
-# 0.5 (eight corrections from 1e-3 to 1e-6 need 0.37), d for the worst: 1e-6
-# for the root mean square.  Above 160 the direct solve is exact to rounding.
+# 2.8e-8 for the faces (0.027); together 2e-7.  From 64 to the limit (300, the
+# mixed form 160) rho may reach 0.5 (eight corrections from 1e-3 to 1e-6 need
+# 0.37), d for the worst: 1e-6 for the root mean square.  Above it the direct
+# solve is exact to rounding.
 @pytest.mark.parametrize("precision", ["fp32", "mixed"])
 @pytest.mark.parametrize("N,K,M", [(4, 64, 24), (6, 64, 12), (8, 64, 12), (10, 32, 16)])
 def test_accepted_groups_are_converged(sl, precision, N, K, M):
@@ -89,10 +90,11 @@ def test_accepted_groups_are_converged(sl, precision, N, K, M):
             direct = s.fallbacks
     L = _conditioning(pb, dW)
     err = np.abs(got[precision] - got["fp64"]).max(-1) / np.abs(got["fp64"]).max(-1)
-    low, mid, high = L <= 64, (L > 64) & (L <= 160), L > 160
+    limit = 300 if precision == "fp32" else 160
+    low, mid, high = L <= 64, (L > 64) & (L <= limit), L > limit
     # the iteration is what is tested: only groups above the limit, and a few
     # near it that need more than its corrections, go to the direct solve
-    assert (L > 160 * 1.001).sum() <= direct[1] <= (L > 160 * 0.999).sum() + 0.05 * mid.sum()
+    assert (L > limit * 1.001).sum() <= direct[1] <= (L > limit * 0.999).sum() + 0.05 * mid.sum()
     assert err[low].max() <= 2e-7
     assert mid.sum() == 0 or np.sqrt((err[mid] ** 2).mean()) <= 1e-6
     assert high.sum() == 0 or err[high].max() <= 2e-7
@@ -119,6 +121,32 @@ def test_fp64_groups_are_refined_to_the_end(sl, orc, N):
     err = np.abs(got - ref).max(-1) / np.abs(ref).max(-1)
     assert direct[1] < 0.5 * L.size  # most groups are the iteration's
     assert err[L <= 4096].max() <= 1e-12
+
+
+# A boundary weight does not hinder the FP64 and FP32 iterations: the null
+# directions of the face rows (one per corner), where the capacitance matrix is
+# w^-2 alone, are filled up before its FP32 inversion.  Rough states at a fifth
+# of the node-gap step (L below 100): nearly every group is iterated.  FP64 as
+# above.  FP32: the last correction is below 1e-6 and rho at most 0.5, in the
+# faces and in the remap: 2e-6.
+@pytest.mark.parametrize("w", [10.0, 30.0])
+@pytest.mark.parametrize("N,K", [(5, 16), (8, 16), (11, 12)])
+def test_boundary_weights_converge(sl, orc, N, K, w):
+    M = 16
+    pb = I.with_(I.config3(M=M, steps=1, K=K, N=N, dt=1e-9), bc_weight=w)
+    q0 = _rough_states(pb)
+    ref = None
+    for prec, tol in (("fp64", 1e-12), ("fp32", 2e-6)):
+        with sl.Solver(pb, prec) as s:
+            s.set_samples(0, q0)
+            pb["dt"] = 0.2 * s.dt_max
+            s.step(dt=pb["dt"], steps=1)
+            got = s.samples().reshape(M, K * K, N * N)
+            direct = s.fallbacks
+        if ref is None:
+            ref = orc.run(pb, state_in=q0, want_states=True, nthreads=16, ns=M)["states"].reshape(got.shape)
+        assert direct[1] <= 0.01 * M * K * K, prec
+        assert (np.abs(got - ref).max(-1) / np.abs(ref).max(-1)).max() <= tol, prec
 
 
 def test_whole_horizon_of_the_64x64_workload(sl):
