@@ -216,12 +216,6 @@ __device__ __forceinline__ void store_state(float2 *Q, long long i, double v)
     const float hi = float(v);
     Q[i] = make_float2(hi, float(v - double(hi)));
 }
-__device__ __forceinline__ double load_state(const double *Q, long long i) { return Q[i]; }
-__device__ __forceinline__ double load_state(const float2 *Q, long long i)
-{
-    const float2 v = Q[i];
-    return double(v.x) + double(v.y);
-}
 
 // One thread per node (e, p), a block per `epb` elements: physical
 // coordinates, drift, sqrt(2D), the initial value, and the divergence of the
@@ -671,7 +665,7 @@ cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, i
                        unsigned int *counts, int nsm, cudaStream_t st)
 {
     if (V == 0) return cudaSuccess;
-    int lp = 5;  // 32 values of up to 383 bins, one of 4096: at most 48 KB
+    int lp = 5;  // 32 values of up to 383 bins, two of 4096: at most 48 KB
     while (lp > 0 && ((size_t(B | 1) << lp) * sizeof(unsigned int)) > 48 * 1024) --lp;
     const size_t smem = (size_t(B | 1) << lp) * sizeof(unsigned int);
     const long long gx = (V + (1LL << lp) - 1) >> lp;
