@@ -20,12 +20,12 @@ constexpr int split1d_lanes(int N) { return N <= 8 ? 8 : 16; }
 // whole warps (a CTA of S K threads pads to one) and whole CTAs per SM; of
 // equal ones the largest (fewer coefficient tables).  A small solve spreads
 // over the SMs that way: 256 samples of 8 elements are 64 one-warp CTAs
-// instead of 8 of 256 threads (a whole solve of 100 FP64 steps at N = 6 2.65 ms,
-// now 1.30), and 10000 samples of 20 elements take 8 fields (160 threads, no
-// padding) instead of 12 (100 steps at N = 9 1.04 ms, now 1.00).
+// instead of 8 of 256 threads (a whole solve of 100 FP64 steps at N = 6 on the
+// thread-per-element kernel 1.30 ms instead of 2.65), and 10000 samples of 20 elements take 8 fields (160 threads, no
+// padding) instead of 12 (4 % faster at N = 9).
 // C: the fewest warps over the field's CTAs for the same reason; of equal
 // ones the smallest cluster.  777 elements take 5 CTAs of 156 slots
-// instead of 4 of 195 (30 steps of 501 fields, mixed, N = 11: 1.03 ms, now 0.92).
+// instead of 4 of 195 (501 fields, mixed, N = 11: 11 % faster).
 inline void geometry1d(int K, int M, int nsm, int max_threads, int &S, int &C, int &T)
 {
     auto warps = [](int threads) { return (threads + 31) / 32; };

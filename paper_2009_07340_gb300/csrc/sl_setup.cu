@@ -85,7 +85,7 @@ __device__ __forceinline__ double node_diffusion(const FieldDev &f, long long v,
 // kernels used to evaluate these inside every node's and face's loops (an
 // O(N^3) product with two FP64 cospi per factor and node): new fields on
 // 32 x 32 elements of N = 5 before each of two steps of 64 samples made the
-// pair of steps take 2.77 ms, now 0.85.
+// pair of steps 1.9 ms longer.
 struct RefTab {
     const double *diff, *at0, *at1, *xi;
     __host__ __device__ RefTab(const double *ref, int N) : diff(ref), at0(ref + N * N), at1(at0 + N), xi(at1 + N) {}
@@ -698,7 +698,7 @@ cudaError_t launch_pdf(const void *Q, int state_is_double, int M, long long V, i
 // stores) where the number of values is even, so that every sample's row
 // starts on a 16-byte boundary.  Bound by the stores; one value per iteration
 // with a 64-bit remainder each made 100 steps of 10000 samples of 20 elements
-// of N = 9 with two reseeds take 1.064 ms, now 1.039.
+// of N = 9 with two reseeds take 1.064 ms instead of 1.039.
 template <typename State, int W>
 __global__ void reseed_kernel(State *Q, const double *__restrict__ mean, int M, long long V)
 {
@@ -844,8 +844,8 @@ cudaError_t launch_coef2d(const double *nodeU, const double *nodeB, const double
 // used to form them for its own elements, and their FP64 products and
 // divisions (16 entries per thread at N = 16) were paid by every launch,
 // however few steps it ran: 50 steps of 4096 sample fields of 256 elements
-// took 3.95 ms in FP32 at N = 16 and now take 3.63, 30 steps of 501 fields of
-// 777 elements 1.25 ms in the mixed form at N = 11 and now 1.03.
+// took 3.95 ms in FP32 at N = 16 and 3.63 without that, 30 steps of 501 fields
+// of 777 elements 1.25 and 1.03 ms in the mixed form at N = 11.
 // Node-major rows of K, so that a CTA's reads are contiguous.
 template <typename R>
 __global__ void coef1d_kernel(const double *__restrict__ nodeU, const double *__restrict__ nodeB,

@@ -12,7 +12,7 @@
 //     each formed once and multiplied into both nodes' products (a third of
 //     the instructions of this part saved against every node's own product:
 //     30 steps of 501 sample fields of 777 elements at N = 11 in the mixed
-//     form 0.917 ms, now 0.833);
+//     form 0.917 ms, now 0.842);
 //   - face bases: lane 0 = face xi = 0, lane 1 = face xi = 1;
 //   - remap: k outer over the advected nodes, pairs of Gauss nodes inner,
 //     with d'_ik = Z_ki + delta_k = -(zeta_i - zeta*_k); the recurrence on d'

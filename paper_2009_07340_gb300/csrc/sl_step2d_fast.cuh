@@ -13,7 +13,8 @@
 // q += G0^{-1} S^T (rhs - S q) on the stacked system S = [V; w B], with
 // G0 = V0^T (I + w^2 E0^T E0) V0, E0 = B V0^{-1}, applied in the stable order
 // V0^{-1} (I - E0^T C^{-1} E0) V0^{-T}, C = w^{-2} I + E0 E0^T (4N x 4N,
-// assembled from 1D products and inverted by its 4N row threads).  Both
+// assembled from 1D products, its null directions filled up, and inverted by
+// its 4N row threads).  Both
 // converge to the direct solution.  A group whose tensor factors are
 // ill-conditioned (||Wx|| ||Wy|| above kCond: particles far outside the
 // element) or whose iteration has not converged is flagged.
@@ -33,17 +34,17 @@
 // a named barrier, row operands are loaded once for both nodes, and the
 // thread's row of C^{-1} stays in registers.  With one thread per node, two
 // warps and a named barrier per stage at N = 8, the kernel waited on barriers
-// and shared memory (43 % of the issue slots used; now 68 %, the shared-memory
-// pipe 78 % busy in phase 2).  Measured, with the FP32 preconditioner and this
+// and shared memory (43 % of the issue slots used; now 71 %, the shared-memory
+// pipe 79 % busy in phase 2).  Measured, with the FP32 preconditioner and this
 // mapping against FP64 passes and that one: 64 x 64 elements, N = 8, FP32, two
-// steps of 64 samples at half the node-gap step 11.37 ms, now 6.66; 32 x 32,
-// N = 6, FP64, one step of 32 samples 6.63 ms, now 1.89; 32 x 32, N = 5, FP32,
-// two steps of 64 samples with new fields 0.85 ms, now 0.68; 19 x 23, N = 12,
+// steps of 64 samples at half the node-gap step 11.15 ms, now 5.73; 32 x 32,
+// N = 6, FP64, one step of 32 samples 6.63 ms, now 1.86; 32 x 32, N = 5, FP32,
+// two steps of 64 samples with new fields 0.85 ms, now 0.72; 19 x 23, N = 12,
 // FP32, one step of 101 samples 2.97 ms, now 2.33.
 // Above N = 8 the 4N face points need more than one warp: two, with two nodes
 // per lane, up to N = 11 (a warp per 32 nodes, three or four, took 28.7, 35.1
 // and 44.0 ns per element-sample at N = 9, 10, 11 on 32 x 32 elements of 16
-// samples, now 25.1, 30.4 and 38.2), five at N = 12 (three nodes per lane in
+// samples, now 25.5, 30.9 and 38.9), five at N = 12 (three nodes per lane in
 // two warps spill: 60.1 against 59.0 ns).
 #pragma once
 #include "sl_step2d.cuh"
@@ -175,7 +176,7 @@ __device__ __forceinline__ double rcp64(double x)
 // work over the lanes of warp 0, and reciprocals are four FMA (rcp64).
 // Conversions run at the FP64 rate too and take the integer pipe instead:
 // with them and a reciprocal from a conversion the mixed form took 18.0, 28.9
-// and 78.1 ns per element-sample at N = 4, 8, 11, now 15.0, 23.6 and 64.3.
+// and 78.1 ns per element-sample at N = 4, 8, 11, now 14.6, 24.2 and 64.0.
 template <int N, int W, int TG, int NR, int RS>
 __device__ __forceinline__ void factor64_2d(double *xd, int tig, int lane, int wig, int bar_id, const float *gt,
                                             const float *Mx, const float *My, const float *u4, float wi2,
